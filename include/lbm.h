@@ -38,7 +38,8 @@
  *     matching LBM_ERR_* code. The state stays readable after such an error.
  *     lbm_init clears the latch. The staged 16-bit step kernel (chosen by
  *     the first lbm_step, see there) bounds each wait for its
- *     asynchronous copies to one second; one that runs out is latched the
+ *     asynchronous copies to one second, and the many-steps launches of small
+ *     lattices each wait between their steps; one that runs out is latched the
  *     same way and returned as LBM_ERR_CUDA, and the steps that followed it
  *     are not valid.
  */
@@ -203,9 +204,11 @@ lbm_status lbm_init_device(lbm_ctx *ctx, const double *U0_dev, const double *u0_
  * register or the shared-memory staged kernel; a few trial steps leave the
  * state untouched, and the fastest is kept for the context's life (the
  * trials take a u*-sized scratch allocation while they run). Until then, and
- * for lbm_step_async, the register kernel runs in static order.
+ * for lbm_step_async, the register kernel runs in static order. Two or more
+ * steps of a small lattice (uniform material, node form of F^b) go in
+ * cooperative launches of up to 64 steps each, with the same results.
  * LBM_STEP16=regs or staged, LBM_DYN=0 or 1 and LBM_DYN_STRIPES=1 or 4 in the
- * environment restrict the choice. */
+ * environment restrict the choice (and keep one launch per step). */
 lbm_status lbm_step(lbm_ctx *ctx, int64_t nsteps);
 
 /* As lbm_step without waiting; check later with lbm_sync. */

@@ -11,6 +11,7 @@
 #include <string>
 #include <vector>
 
+#include "lbm_edges.cuh"
 #include "lbm_internal.h"
 
 using namespace tlv;
@@ -73,7 +74,7 @@ lbm_status map_flags(lbm_ctx *c, int flags)
     if (flags & ST_NONFINITE) return fail(c, LBM_ERR_NONFINITE, "the state became non-finite");
     if (flags & ST_BAD_J) return fail(c, LBM_ERR_NONPOSITIVE_J, "a node reached J = det F <= 0");
     if (flags & ST_NEWTON) return fail(c, LBM_ERR_NEWTON, "a traction-edge Newton solve did not converge");
-    if (flags & ST_STALL) return fail(c, LBM_ERR_CUDA, "a step kernel's wait for its bulk copies exceeded its time bound");
+    if (flags & ST_STALL) return fail(c, LBM_ERR_CUDA, "a step kernel's wait (for its bulk copies, or between the steps of one launch) exceeded its time bound");
     return LBM_OK;
 }
 
@@ -196,6 +197,25 @@ lbm_status record(lbm_ctx *c, std::vector<cudaEvent_t> &v)
     return LBM_OK;
 }
 
+// `len` steps from a (a.fin and a.fout the two buffers) in one cooperative
+// launch; the edges' data of the steps go along as an argument
+template <typename T>
+cudaError_t launch_multi(lbm_ctx *c, StepArgs<T> a, int len)
+{
+    StepTimes<T> tab;
+    for (int k = 0; k < len; ++k)
+        for (int e = 0; e < 4; ++e) {
+            tab.g[k][e] = ctx_time_factor(c, e, c->step + k);
+            tab.val[k][e] = edge_val<T>(c->edge[e].value, tab.g[k][e], a.c);
+        }
+    unsigned *count = c->d_ctr + 2 * DYN_SET_WORDS;
+    cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned), c->st);
+    if (e != cudaSuccess) return e;
+    void *params[] = {&a, &tab, &len, &count};
+    return cudaLaunchCooperativeKernel(c->multi_fn, dim3((unsigned)c->multi_grid), dim3((unsigned)c->multi_block),
+                                       params, 0, c->st);
+}
+
 // In the node form of F^b every ghost value depends only on its own boundary
 // node, so the step kernel writes the next step's ghosts itself (fused) and
 // the separate ghost kernel runs only when they are stale. The extrapolated
@@ -205,7 +225,23 @@ lbm_status do_step(lbm_ctx *c, int64_t nsteps)
 {
     const bool prof = c->prof && (c->ev_step.size() < 200000);
     const bool fuse = c->cfg.fb_mode == LBM_FB_NODE;
-    for (int64_t i = 0; i < nsteps; ++i) {
+    int64_t i = 0;
+    // a small lattice: up to MULTI_STEPS steps per launch (launches are
+    // counted and timed one step each when profiling)
+    if (c->multi_fn && !c->prof && nsteps > 1) {
+        if (c->ghosts_dirty) {
+            CK(c, launch_ghosts(c->cfg.storage, edge_args(c, c->cur), c->edge_blk_end[3], c->st));
+            c->ghosts_dirty = false;
+        }
+        for (; nsteps - i > 1;) {
+            const int len = (int)std::min<int64_t>(nsteps - i, MULTI_STEPS);
+            CK(c, launch_multi(c, step_args<T>(c, c->cur), len));
+            c->cur ^= len & 1;
+            c->step += len;
+            i += len;
+        }
+    }
+    for (; i < nsteps; ++i) {
         if (!fuse || c->ghosts_dirty) {
             const EdgeArgs ea = edge_args(c, c->cur);
             if (prof && record(c, c->ev_edge) != LBM_OK) return LBM_ERR_CUDA;
@@ -402,6 +438,42 @@ static void drop_material_field(lbm_ctx *c)
     c->m.lam_ratio = 0.0;
 }
 
+// The many-steps kernel (k_multi) takes lattices of up to this many nodes: a
+// step of a larger one lasts longer than its launch, and the step kernels'
+// wider loads win. Both sides, us per step (own launches / k_multi): FP64
+// 384^2 periodic 41 / 33, 512^2 clamped 105 / 118; FP32 800^2 periodic
+// 29 / 23, 1024^2 clamped 45 / 41; BF16 700 x 500 clamped 19 / 12, 1024^2
+// clamped 30 / 28.6; FP16 1024 x 512 periodic 12.2 / 12.0.
+static long long multi_nodes(int storage)
+{
+    return storage == STORE_F64 ? 160 << 10 : storage == STORE_F32 ? 1 << 20 : 640 << 10;
+}
+
+static void set_multi(lbm_ctx *c, int sms)
+{
+    c->multi_fn = nullptr;
+    if (c->cfg.fb_mode != LBM_FB_NODE || c->m.mufield) return;
+    if ((long long)c->L.nx * c->L.ny > multi_nodes(c->cfg.storage)) return;
+    // the environment asks for one of the step kernels
+    if (dyn_env_choice() >= 0 || stripes_env_choice() >= 0 || step16_env_choice() >= 0) return;
+    int coop = 0, per_sm = 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->cfg.device) != cudaSuccess || !coop) return;
+    const void *fn = nullptr;
+    switch (c->cfg.storage) {
+    case STORE_F64: fn = multi_kernel_f64(c->m.law); break;
+    case STORE_BF16: fn = multi_kernel_bf16(c->m.law); break;
+    case STORE_F16: fn = multi_kernel_f16(c->m.law); break;
+    default: fn = multi_kernel_f32(c->m.law); break;
+    }
+    // few tasks: one warp to a block, so that they spread over the SMs
+    const long long tasks = (long long)c->L.ny * ((c->L.nx + 31) / 32);
+    const int warps = (int)std::min<long long>(MULTI_WARPS, std::max<long long>(1, (tasks + sms - 1) / sms));
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * warps, 0) != cudaSuccess || per_sm < 1) return;
+    c->multi_fn = fn;
+    c->multi_block = 32 * warps;
+    c->multi_grid = (int)std::min<long long>((tasks + warps - 1) / warps, (long long)per_sm * sms);
+}
+
 static lbm_status set_step_grid(lbm_ctx *c)
 {
     int sms = 0;
@@ -413,6 +485,7 @@ static lbm_status set_step_grid(lbm_ctx *c)
     long long g = (long long)(sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
     if (g > needed) g = needed;
     c->grid_step = (int)(g < 1 ? 1 : g);
+    set_multi(c, sms > 0 ? sms : 1);
     return LBM_OK;
 }
 
@@ -505,8 +578,8 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out)
     CKC(cudaMalloc((void **)&c->ustar, ubytes));
     CKC(cudaMalloc((void **)&c->d_status, sizeof(int)));
     CKC(cudaMalloc((void **)&c->d_diag, (size_t)(diag_blocks(c->L) * 10 + 10) * sizeof(double)));
-    CKC(cudaMalloc((void **)&c->d_ctr, 2 * DYN_SET_WORDS * sizeof(unsigned)));
-    CKC(cudaMemset(c->d_ctr, 0, 2 * DYN_SET_WORDS * sizeof(unsigned)));
+    CKC(cudaMalloc((void **)&c->d_ctr, CTR_WORDS * sizeof(unsigned)));
+    CKC(cudaMemset(c->d_ctr, 0, CTR_WORDS * sizeof(unsigned)));
     c->dyn = tlv::dyn_env_choice() == 1 ? DYN_STRIPES : 0;  // until the first lbm_step chooses
     CKC(cudaMemsetAsync(c->f[0], 0, fbytes, c->st));
     CKC(cudaMemsetAsync(c->f[1], 0, fbytes, c->st));

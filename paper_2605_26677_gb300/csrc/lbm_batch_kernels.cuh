@@ -32,7 +32,7 @@ __device__ __forceinline__ void batch_loop(const BatchList &b, int *off, int *xq
     auto proc = [&](int x, int y, int mm) {
         const StepArgs<T> &a = args[mm];
         unsigned f = 0;
-        xedge_node<LAW, S>(a, x, y, f);
+        xedge_node<LAW, S>(a, step_io(a), x, y, f);
         if (f) atomicOr(a.status, (int)f);
     };
     int m = 0;
@@ -53,9 +53,9 @@ __device__ __forceinline__ void batch_loop(const BatchList &b, int *off, int *xq
         unsigned flags = 0;
         XPend xp{-1, 0};
         if constexpr (PACKED)
-            step16_task<S, LAW, V, true>(a, task - off[m], lane, flags);
+            step16_task<S, LAW, V, true>(a, step_io(a), task - off[m], lane, flags);
         else
-            step_task<S, LAW, V, true, false, false, XQ>(a, task - off[m], lane, flags, &xp);
+            step_task<S, LAW, V, true, false, false, XQ>(a, step_io(a), task - off[m], lane, flags, &xp);
         flags = __reduce_or_sync(FULL_MASK, flags);
         if (flags && lane == 0) atomicOr(a.status, (int)flags);
         if constexpr (XQ) xq_push(q, xp, m, lane, proc);

@@ -199,6 +199,27 @@ struct StepArgs {
 constexpr int DYN_STRIPES = 4;
 constexpr int DYN_CTR_STRIDE = 64;
 constexpr int DYN_SET_WORDS = DYN_STRIPES * DYN_CTR_STRIDE;
+// a context's counters: the two sets and the grid barrier's count (k_multi)
+constexpr int CTR_WORDS = 2 * DYN_SET_WORDS + DYN_CTR_STRIDE;
+
+// Edge data at a boundary node (see edge_val): v_D or the traction, and the
+// same over c
+template <typename R>
+struct EdgeVal {
+    R v[2], vc[2];
+};
+
+// Edge data of the steps of one many-steps launch (a kernel argument): the
+// time factors, and the values of edges without a profile
+constexpr int MULTI_STEPS = 64;
+constexpr int MULTI_WARPS = 8;  // warps per block at most (4: more blocks meet at the barrier,
+                                // 512^2 FP32 8.7 against 8.0 us a step; 16: 7.7, but FP64 512^2 138
+                                // against 113)
+template <typename R>
+struct StepTimes {
+    double g[MULTI_STEPS][4];
+    EdgeVal<R> val[MULTI_STEPS][4];
+};
 
 // A batch of lattices for one persistent launch
 constexpr int BATCH_MAX_MEMBERS = 4096;

@@ -147,31 +147,61 @@ __device__ bool traction_newton(int e, R G[4], const R Tb[2], const LawP<R> &m)
     return fmax(fabs(r[0]), fabs(r[1])) <= newton_tol<R>(tmax, mus, gmax);
 }
 
+// The Newton solve of a law with a logarithm in FP64, compiled on its own:
+// inlined, the compiler contracts its products differently from kernel to
+// kernel, and a run's last bit would depend on which kernel took its steps.
+template <int LAW, typename R>
+__device__ __noinline__ bool traction_newton_call(int e, R G[4], R T0, R T1, const LawP<R> &m)
+{
+    const R Tb[2] = {T0, T1};
+    return traction_newton<LAW, R>(e, G, Tb, m);
+}
+
+// Edge data of one boundary node at t^n + dt/2 in the compute type, and the
+// same divided by c. On an edge without a profile they are the same for
+// every node: formed once on the host they spare each boundary lane two FP64
+// products, two conversions and the divisions.
+template <typename R>
+__host__ __device__ __forceinline__ EdgeVal<R> edge_val(const double value[2], double g, R c)
+{
+    EdgeVal<R> v;
+    v.v[0] = (R)(value[0] * g);
+    v.v[1] = (R)(value[1] * g);
+    v.vc[0] = v.v[0] / c;
+    v.vc[1] = v.v[1] / c;
+    return v;
+}
+
 // Ghost value of a velocity or traction edge in the node form. fo: f*_{-d}
 // at the boundary node (offsets); U: (v, G) at the node at t^n; val: edge data
 // at t^n + dt/2. Writes out[6]; sets ST_NEWTON in flags on failure.
 template <int LAW, typename R>
-__device__ __forceinline__ void edge_ghost(int e, int kind, const R fo[6], const R U[6], const double val[2],
-                                           R c, const LawP<R> &m, R out[6], unsigned &flags)
+__device__ __forceinline__ void edge_ghost(int e, int kind, const R fo[6], const R U[6], const EdgeVal<R> &val,
+                                           const LawP<R> &m, R out[6], unsigned &flags)
 {
     const R N0 = (e == EDGE_LEFT) ? R(-1) : (e == EDGE_RIGHT) ? R(1) : R(0);
     const R N1 = (e == EDGE_BOTTOM) ? R(-1) : (e == EDGE_TOP) ? R(1) : R(0);
-    const R v0 = (R)val[0], v1 = (R)val[1];
+    const R v0 = val.v[0], v1 = val.v[1], v0c = val.vc[0], v1c = val.vc[1];
     if (kind == BC_VELOCITY) {
         // Eq. (24): D = diag(-1,-1,1,1,1,1), S = (vD/2, N1 vD1/c, N2 vD1/c, N1 vD2/c, N2 vD2/c)
         out[0] = -fo[0] + R(0.5) * v0;
         out[1] = -fo[1] + R(0.5) * v1;
-        out[2] = fo[2] + N0 * v0 / c;
-        out[3] = fo[3] + N1 * v0 / c;
-        out[4] = fo[4] + N0 * v1 / c;
-        out[5] = fo[5] + N1 * v1 / c;
+        out[2] = fo[2] + N0 * v0c;
+        out[3] = fo[3] + N1 * v0c;
+        out[4] = fo[4] + N0 * v1c;
+        out[5] = fo[5] + N1 * v1c;
     } else {
         // Eq. (25): D = diag(1,1,-1,-1,-1,-1), S = (T/c, F^b/2)
         R G[4] = {U[2], U[3], U[4], U[5]};
         const R Tb[2] = {v0, v1};
-        if (!traction_newton<LAW, R>(e, G, Tb, m)) flags |= ST_NEWTON;
-        out[0] = fo[0] + v0 / c;
-        out[1] = fo[1] + v1 / c;
+        bool ok;
+        if constexpr (sizeof(R) == 8 && LAW >= LAW_LOGNH)
+            ok = traction_newton_call<LAW, R>(e, G, v0, v1, m);
+        else
+            ok = traction_newton<LAW, R>(e, G, Tb, m);
+        if (!ok) flags |= ST_NEWTON;
+        out[0] = fo[0] + v0c;
+        out[1] = fo[1] + v1c;
 #pragma unroll
         for (int m = 0; m < 4; ++m) out[2 + m] = -fo[2 + m] + R(0.5) * G[m];
     }

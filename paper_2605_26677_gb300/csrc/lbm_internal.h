@@ -73,6 +73,8 @@ struct lbm_ctx {
     bool initialized = false;
     bool ghosts_dirty = true;  // ghost cells of f[cur] must be rebuilt before the next step
     int grid_step = 1;
+    const void *multi_fn = nullptr;  // many-steps kernel of a small lattice (set_multi), or nullptr
+    int multi_block = 0, multi_grid = 0;
     int edge_blk_end[4] = {0, 0, 0, 0};
     std::string err;
     bool prof = false;
@@ -108,6 +110,12 @@ cudaError_t launch_edges(int storage, const EdgeArgs &a, int grid, cudaStream_t 
 cudaError_t launch_ghosts(int storage, const EdgeArgs &a, int grid, cudaStream_t st);
 int step_blocks_per_sm(int storage, int law);
 int step_vec(int storage);
+
+// lbm_multi_<type>.cu: the many-steps kernel
+const void *multi_kernel_f64(int law);
+const void *multi_kernel_f32(int law);
+const void *multi_kernel_bf16(int law);
+const void *multi_kernel_f16(int law);
 
 // lbm_aux.cu
 struct InitArgs {

@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(128, Stage16<NS>::MIN_BLOCKS) k_step16s(const 
                 for (int e = 0; e < V; ++e) u[c].v[e] += a.dt * (double)vel[c][e];
                 *reinterpret_cast<PD *>(a.ustar + c * a.L.uplane + urow) = u[c];
             }
-            if (FUSE) lane_ghosts<LAW, S, V>(a, reinterpret_cast<S *>(fout), row, x0, y, flags);
+            if (FUSE) lane_ghosts<LAW, S, V>(a, a.gdev, reinterpret_cast<S *>(fout), row, x0, y, flags);
         }
     }
     flags = __reduce_or_sync(FULL_MASK, flags);

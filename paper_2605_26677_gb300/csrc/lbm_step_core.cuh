@@ -15,6 +15,19 @@ struct alignas(sizeof(T) * N) Pack {
 
 #define FULL_MASK 0xffffffffu
 
+// What changes from one step of a launch to the next: the population buffers
+// and the edges' time factors (nullptr: StepArgs::g)
+struct StepIO {
+    const void *fin;
+    void *fout;
+    const double *gdev;
+};
+template <typename T>
+__device__ __forceinline__ StepIO step_io(const StepArgs<T> &a)
+{
+    return StepIO{a.fin, a.fout, a.gdev};
+}
+
 // x is NaN or infinite: all exponent bits set, tested on the integer pipe
 // (the FP64 pipe is the FP64 step's bottleneck)
 __device__ __forceinline__ bool nonfinite(double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; }
@@ -147,9 +160,10 @@ __device__ __forceinline__ void collide_node(T f[4][6], const StepArgs<T> &a, co
 // row (plane 3, y = ny), left ghost column (plane 0, x = -1), right ghost
 // column (plane 2, x = nx), with the edge data of the step that will pull
 // these values.
-template <int LAW, typename S, typename T, bool SKIP_X = false>
-__device__ __forceinline__ void node_ghosts(const T f[4][6], int x, int y, const StepArgs<T> &a, const LawP<T> &m,
-                                            S *fout, unsigned &flags)
+// ev(e, s): the edge data (EdgeVal) of position s of edge e.
+template <int LAW, typename S, typename T, typename EV>
+__device__ __forceinline__ void node_ghosts(const T f[4][6], int x, int y, const StepArgs<T> &a, EV &&ev,
+                                            const LawP<T> &m, S *fout, unsigned &flags)
 {
     const int nx = a.L.nx, ny = a.L.ny;
     auto put = [&](int e, int gx, int gy, const T val[6]) {
@@ -161,9 +175,7 @@ __device__ __forceinline__ void node_ghosts(const T f[4][6], int x, int y, const
     auto rule = [&](int e, int s, int gx, int gy) {
         T U[6], out[6];
         state_from_fstar(f[0], f[1], f[2], f[3], a.hdtb1, a.hdtb2, U);
-        const double g = (a.gdev ? a.gdev[e] : a.g[e]) * (a.profile[e] ? a.profile[e][s] : 1.0);
-        const double val[2] = {a.value[e][0] * g, a.value[e][1] * g};
-        edge_ghost<LAW, T>(e, a.kind[e], f[edge_dout(e)], U, val, a.c, m, out, flags);
+        edge_ghost<LAW, T>(e, a.kind[e], f[edge_dout(e)], U, ev(e, s), m, out, flags);
         put(e, gx, gy, out);
     };
     if (a.kind[EDGE_BOTTOM] == BC_PERIODIC) {
@@ -176,7 +188,7 @@ __device__ __forceinline__ void node_ghosts(const T f[4][6], int x, int y, const
     if (a.kind[EDGE_LEFT] == BC_PERIODIC) {
         if (x == nx - 1) put(EDGE_LEFT, -1, y, f[0]);
         if (x == 0) put(EDGE_RIGHT, nx, y, f[2]);
-    } else if (!SKIP_X) {
+    } else {
         if (x == 0) rule(EDGE_LEFT, y, -1, y);
         if (x == nx - 1) rule(EDGE_RIGHT, y, nx, y);
     }
@@ -248,10 +260,12 @@ __device__ __forceinline__ void xq_push(XQueue &q, const XPend &xp, int m, int l
 }
 
 template <int LAW, typename S, bool MATF = false>
-__device__ __forceinline__ void xedge_node(const StepArgs<typename Prec<S>::R> &a, int x, int y, unsigned &flags)
+__device__ __forceinline__ void xedge_node(const StepArgs<typename Prec<S>::R> &a, const StepIO &io, int x, int y,
+                                           unsigned &flags)
 {
     using T = typename Prec<S>::R;
-    S *fout = static_cast<S *>(a.fout);
+    S *fout = static_cast<S *>(io.fout);
+    const double *gdev = io.gdev;
     const long long row = (long long)(y + 1) * a.L.pitch + a.L.xoff + x;
     T fq[4][6];
 #pragma unroll
@@ -271,9 +285,8 @@ __device__ __forceinline__ void xedge_node(const StepArgs<typename Prec<S>::R> &
     for (int side = 0; side < 2; ++side) {
         const int e = side == 0 ? EDGE_LEFT : EDGE_RIGHT;
         if ((side == 0 && x != 0) || (side == 1 && x != nx - 1)) continue;
-        const double g = (a.gdev ? a.gdev[e] : a.g[e]) * (a.profile[e] ? a.profile[e][y] : 1.0);
-        const double val[2] = {a.value[e][0] * g, a.value[e][1] * g};
-        edge_ghost<LAW, T>(e, a.kind[e], fq[edge_dout(e)], U, val, a.c, m, out, flags);
+        const double g = (gdev ? gdev[e] : a.g[e]) * (a.profile[e] ? a.profile[e][y] : 1.0);
+        edge_ghost<LAW, T>(e, a.kind[e], fq[edge_dout(e)], U, edge_val<T>(a.value[e], g, a.c), m, out, flags);
         S *dst = fout + (long long)(edge_dmiss(e) * 6) * a.L.plane + (long long)(y + 1) * a.L.pitch + a.L.xoff +
                  (side == 0 ? -1 : nx);
 #pragma unroll
@@ -301,8 +314,8 @@ __device__ __forceinline__ void task_coords(int task, int nseg, int ny, int &y, 
 // of the streaming loop, and it sees exactly the values the ghost-refresh
 // kernel would read.
 template <int LAW, typename S, int VEC, bool MATF = false, bool XQ = false>
-__device__ __forceinline__ void lane_ghosts(const StepArgs<typename Prec<S>::R> &a, S *fout, long long row, int x0,
-                                            int y, unsigned &flags, XPend *xp = nullptr)
+__device__ __forceinline__ void lane_ghosts(const StepArgs<typename Prec<S>::R> &a, const double *gdev, S *fout,
+                                            long long row, int x0, int y, unsigned &flags, XPend *xp = nullptr)
 {
     using T = typename Prec<S>::R;
     const int nx = a.L.nx, ny = a.L.ny;
@@ -332,7 +345,10 @@ __device__ __forceinline__ void lane_ghosts(const StepArgs<typename Prec<S>::R> 
             m.mu = a.mufield[(long long)y * a.L.upitch + x];
             m.lam = a.lam_ratio * m.mu;
         }
-        node_ghosts<LAW, S, T>(fq, x, y, a, m, fout, flags);
+        auto ev = [&](int ed, int s) {
+            return edge_val<T>(a.value[ed], (gdev ? gdev[ed] : a.g[ed]) * (a.profile[ed] ? a.profile[ed][s] : 1.0), a.c);
+        };
+        node_ghosts<LAW, S, T>(fq, x, y, a, ev, m, fout, flags);
     }
 }
 
@@ -341,7 +357,7 @@ __device__ __forceinline__ void lane_ghosts(const StepArgs<typename Prec<S>::R> 
 // NOQ: no displacement quadrature (states recomputed only for their
 // populations, as the adjoint's checkpoint segments are).
 template <typename S, int LAW, int VEC, bool FUSE, bool MATF = false, bool NOQ = false, bool XQ = false>
-__device__ __forceinline__ void step_task(const StepArgs<typename Prec<S>::R> &a, int task, int lane,
+__device__ __forceinline__ void step_task(const StepArgs<typename Prec<S>::R> &a, const StepIO &io, int task, int lane,
                                           unsigned &flags, XPend *xp = nullptr)
 {
     using T = typename Prec<S>::R;  // compute type
@@ -352,8 +368,8 @@ __device__ __forceinline__ void step_task(const StepArgs<typename Prec<S>::R> &a
     const int nseg = (nx + segw - 1) / segw;
     const long long plane = a.L.plane;
     const int pitch = a.L.pitch;
-    const S *__restrict__ fin = static_cast<const S *>(a.fin);
-    S *__restrict__ fout = static_cast<S *>(a.fout);
+    const S *__restrict__ fin = static_cast<const S *>(io.fin);
+    S *__restrict__ fout = static_cast<S *>(io.fout);
     {
         int y, seg;
         task_coords(task, nseg, a.L.ny, y, seg);
@@ -440,7 +456,7 @@ __device__ __forceinline__ void step_task(const StepArgs<typename Prec<S>::R> &a
                     *reinterpret_cast<PD *>(a.ustar + c * a.L.uplane + urow) = u;
                 }
             }
-            if (FUSE) lane_ghosts<LAW, S, VEC, MATF, XQ>(a, fout, row, x0, y, flags, xp);
+            if (FUSE) lane_ghosts<LAW, S, VEC, MATF, XQ>(a, io.gdev, fout, row, x0, y, flags, xp);
         }
     }
 }
@@ -474,7 +490,7 @@ struct Words {
 };
 
 template <typename S, int LAW, int V, bool FUSE, bool MATF = false>
-__device__ __forceinline__ void step16_task(const StepArgs<float> &a, int task, int lane, unsigned &flags)
+__device__ __forceinline__ void step16_task(const StepArgs<float> &a, const StepIO &io, int task, int lane, unsigned &flags)
 {
     constexpr int W = V / 2;  // 32-bit words per vector
     using WV = Words<W>;
@@ -485,8 +501,8 @@ __device__ __forceinline__ void step16_task(const StepArgs<float> &a, int task, 
     const int nseg = (nx + segw - 1) / segw;
     const long long plane = a.L.plane;
     const int pitch = a.L.pitch;
-    const unsigned short *__restrict__ fin = static_cast<const unsigned short *>(a.fin);
-    unsigned short *__restrict__ fout = static_cast<unsigned short *>(a.fout);
+    const unsigned short *__restrict__ fin = static_cast<const unsigned short *>(io.fin);
+    unsigned short *__restrict__ fout = static_cast<unsigned short *>(io.fout);
     auto ldv = [&](const unsigned short *p) {
         WV r;
         if constexpr (W == 2) {
@@ -610,7 +626,7 @@ __device__ __forceinline__ void step16_task(const StepArgs<float> &a, int task, 
                     for (int e = 0; e < 4; ++e) u[c][h].v[e] += a.dt * (double)vel[c][4 * h + e];
                     *reinterpret_cast<PD *>(a.ustar + c * a.L.uplane + urow + 4 * h) = u[c][h];
                 }
-            if (FUSE) lane_ghosts<LAW, S, V, MATF>(a, reinterpret_cast<S *>(fout), row, x0, y, flags);
+            if (FUSE) lane_ghosts<LAW, S, V, MATF>(a, io.gdev, reinterpret_cast<S *>(fout), row, x0, y, flags);
         }
     }
 }

@@ -41,10 +41,11 @@ __global__ void __launch_bounds__(128) k_step(const StepArgs<typename Prec<S>::R
     constexpr bool XQ = FUSE && sizeof(S) == 8;
     __shared__ int xq[XQ ? 4 * 3 * XQ_CAP : 1];
     XQueue q = XQ ? xq_make(xq) : XQueue{nullptr, nullptr, nullptr, 0};
-    auto proc = [&](int x, int y, int) { xedge_node<LAW, S, MATF>(a, x, y, flags); };
+    const StepIO io = step_io(a);
+    auto proc = [&](int x, int y, int) { xedge_node<LAW, S, MATF>(a, io, x, y, flags); };
     auto run = [&](int task) {
         XPend xp{-1, 0};
-        step_task<S, LAW, VEC, FUSE, MATF, NOQ, XQ>(a, task, lane, flags, &xp);
+        step_task<S, LAW, VEC, FUSE, MATF, NOQ, XQ>(a, io, task, lane, flags, &xp);
         if constexpr (XQ) xq_push(q, xp, 0, lane, proc);
     };
     if constexpr (DYN)
@@ -69,9 +70,9 @@ __global__ void __launch_bounds__(128, 4) k_step16(const StepArgs<float> a)
     unsigned flags = 0;
     if constexpr (DYN > 0)
         dyn_tasks<DYN>(a.ctr, a.ctr_next, ntask, lane,
-                       [&](int task) { step16_task<S, LAW, V, FUSE, MATF>(a, task, lane, flags); });
+                       [&](int task) { step16_task<S, LAW, V, FUSE, MATF>(a, step_io(a), task, lane, flags); });
     else
-        for (int task = gw; task < ntask; task += nw) step16_task<S, LAW, V, FUSE, MATF>(a, task, lane, flags);
+        for (int task = gw; task < ntask; task += nw) step16_task<S, LAW, V, FUSE, MATF>(a, step_io(a), task, lane, flags);
     flags = __reduce_or_sync(FULL_MASK, flags);
     if (flags && lane == 0) atomicOr(a.status, (int)flags);
 }
@@ -117,11 +118,10 @@ __global__ void __launch_bounds__(128) k_ghosts(const EdgeArgs a)
     state_from_fstar(fq[0], fq[1], fq[2], fq[3], (T)a.hdtb1, (T)a.hdtb2, U);
 #pragma unroll
     for (int k = 0; k < 6; ++k) fo[k] = fq[md][k];
-    double val[2];
-    edge_value(E, s, a.g[e], val);
     unsigned flags = 0;
     const LawP<T> m = law_cast<T>(law_at(a.m, (long long)yb * a.L.nx + xb));
-    edge_ghost<LAW, T>(e, E.kind, fo, U, val, (T)a.c, m, out, flags);
+    edge_ghost<LAW, T>(e, E.kind, fo, U, edge_val<T>(E.value, a.g[e] * (E.profile ? E.profile[s] : 1.0), (T)a.c), m, out,
+                       flags);
     if (flags) atomicOr(a.status, (int)flags);
 #pragma unroll
     for (int k = 0; k < 6; ++k) f[idx(d, k, gx, gy)] = to_store<S>(out[k]);

@@ -294,7 +294,7 @@ lbm_status lbm_adjoint_create(lbm_ctx *c, int64_t nsteps, int32_t checkpoint_eve
     a->nsteps = nsteps;
     a->K = checkpoint_every > 0 ? checkpoint_every
                                 : std::max(1, (int)std::ceil(std::sqrt((double)std::max<long long>(nsteps, 1))));
-    a->fbytes = (size_t)24 * (size_t)c->L.plane * c->eb;
+    a->fbytes = (size_t)c->L.total * c->eb;
     // dynamic claims on one counter: backward / forward 1.656 at 1024^2
     // against 1.706 in static order and 1.696 over four stripes
     a->dyn = (c->cfg.storage == LBM_STORE_F32) ? adj_dyn_choice(1) : 0;

@@ -544,6 +544,17 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out)
     c->L.xoff = line;
     c->L.pitch = (int)round_up((long long)line + cfg->nx + vec, line);
     c->L.plane = (long long)(cfg->ny + 2) * c->L.pitch;
+    c->L.total = 24 * c->L.plane;
+    // The 24 planes of a row lie one after another, so that a task's loads
+    // and stores stay within a few pages instead of one page per plane
+    // (us per step, plane after plane / row after row: 8192^2 FP32 2201 /
+    // 2145, 4096 x 2048 clamped FP32 284.5 / 278.8, BF16 168.5 / 163.5,
+    // 4096^2 FP16 324 / 314). A row whose 24 planes exceed the pitch that a
+    // 2-D copy can take keeps plane after plane.
+    if (24LL * c->L.pitch * c->eb <= INT32_MAX) {
+        c->L.plane = c->L.pitch;
+        c->L.pitch *= 24;
+    }
     c->L.upitch = (int)round_up((long long)cfg->nx + 4, 16);
     c->L.uplane = (long long)cfg->ny * c->L.upitch;
     for (int e = 0; e < 4; ++e) {
@@ -555,7 +566,7 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out)
         blk += (edge_len(c, e) + 127) / 128;
         c->edge_blk_end[e] = blk;
     }
-    const size_t fbytes = (size_t)24 * (size_t)c->L.plane * c->eb;
+    const size_t fbytes = (size_t)c->L.total * c->eb;
     const size_t ubytes = (size_t)2 * (size_t)c->L.uplane * sizeof(double);
 
     cudaError_t e = cudaSetDevice(cfg->device);
@@ -1033,7 +1044,7 @@ lbm_status lbm_init(lbm_ctx *c, const double *U0, const double *u0, int32_t orde
     // initialization writes f[0] and the first step overwrites f[1], and its
     // 24 planes hold U0's 6 N doubles in every storage type (u0's 2 N too,
     // except with 16-bit storage, where u0 gets an allocation of its own).
-    const size_t fbytes = (size_t)24 * c->L.plane * c->eb;
+    const size_t fbytes = (size_t)c->L.total * c->eb;
     double *dU = static_cast<double *>(c->f[1]), *du = nullptr;
     bool du_owned = false;
     cudaError_t e = cudaSuccess;

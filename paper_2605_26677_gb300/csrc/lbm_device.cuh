@@ -2,8 +2,8 @@
 // physics of the total-Lagrangian vectorial D2Q4x6 LBM (Feng & Chu).
 //
 // Population storage (both buffers): 24 planes p = q*6 + k (direction q of
-// Sec. 3.1, state component k of Eq. 5), each (ny + 2) rows x pitch elements.
-// Row 0 and row ny + 1 are ghost rows (y = -1, y = ny); column xoff - 1 and
+// Sec. 3.1, state component k of Eq. 5) of ny + 2 rows, the 24 planes' copies
+// of a row one after another. Row 0 and row ny + 1 are ghost rows (y = -1, y = ny); column xoff - 1 and
 // column xoff + nx are ghost columns (x = -1, x = nx). Node (x, y) lives at
 //   p * plane + (y + 1) * pitch + xoff + x.
 // xoff is 128 bytes, so every row of real nodes starts on a 128-byte line.
@@ -83,8 +83,9 @@ enum { FB_NODE = 0, FB_EXTRAP2 = 1 };
 enum { ST_BAD_J = 1, ST_NEWTON = 2, ST_NONFINITE = 4, ST_STALL = 8 };  // ST_STALL: a bounded wait gave up
 
 struct Layout {
-    long long plane;  // elements per population plane
-    int pitch;        // elements per row
+    long long plane;  // elements from a row's plane p to its plane p + 1
+    long long total;  // elements of a population buffer
+    int pitch;        // elements from a plane's row to its next
     int xoff;         // column of node x = 0
     int nx, ny;
     long long uplane; // doubles per u* plane

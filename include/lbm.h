@@ -206,7 +206,9 @@ lbm_status lbm_init_device(lbm_ctx *ctx, const double *U0_dev, const double *u0_
  * trials take a u*-sized scratch allocation while they run). Until then, and
  * for lbm_step_async, the register kernel runs in static order. Two or more
  * steps of a small lattice (uniform material, node form of F^b) go in
- * cooperative launches of up to 64 steps each, with the same results.
+ * cooperative launches of up to 64 steps each, those of a larger FP32 lattice
+ * in launches of two steps, with the same results; such calls need no
+ * variant and leave the choice to a later one.
  * LBM_STEP16=regs or staged, LBM_DYN=0 or 1 and LBM_DYN_STRIPES=1 or 4 in the
  * environment restrict the choice (and keep one launch per step). */
 lbm_status lbm_step(lbm_ctx *ctx, int64_t nsteps);

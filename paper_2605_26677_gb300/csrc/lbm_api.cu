@@ -197,6 +197,13 @@ lbm_status record(lbm_ctx *c, std::vector<cudaEvent_t> &v)
     return LBM_OK;
 }
 
+// Whether nsteps steps go several to a launch (k_multi, k_pair). Launches are
+// counted and timed one step each when profiling.
+bool grouped_steps(const lbm_ctx *c, int64_t nsteps)
+{
+    return (c->multi_fn || c->pair_grid) && !c->prof && nsteps > 1;
+}
+
 // `len` steps from a (a.fin and a.fout the two buffers) in one cooperative
 // launch; the edges' data of the steps go along as an argument
 template <typename T>
@@ -216,6 +223,38 @@ cudaError_t launch_multi(lbm_ctx *c, StepArgs<T> a, int len)
                                        params, 0, c->st);
 }
 
+// 2 `pairs` steps with the two-step kernel
+cudaError_t do_pairs(lbm_ctx *c, int64_t pairs)
+{
+    if (c->ghosts_dirty) {
+        const cudaError_t e = launch_ghosts(c->cfg.storage, edge_args(c, c->cur), c->edge_blk_end[3], c->st);
+        if (e != cudaSuccess) return e;
+        c->ghosts_dirty = false;
+    }
+    if (xper(c)) {
+        // each pair leaves these columns for the next; the first one's input may come from elsewhere
+        const cudaError_t e = launch_wide_f32(c->f[c->cur], c->L, c->st);
+        if (e != cudaSuccess) return e;
+    }
+    for (int64_t i = 0; i < pairs; ++i) {
+        PairArgs<float> p;
+        p.a = step_args<float>(c, c->cur);
+        for (int e = 0; e < 4; ++e) {
+            p.g1[e] = p.a.g[e];
+            p.v1[e] = edge_val<float>(p.a.value[e], p.g1[e], p.a.c);
+            p.a.g[e] = ctx_time_factor(c, e, c->step + 1);
+        }
+        p.a.ctr2 = c->d_ctr;
+        p.nstrip = c->pair_strips;
+        p.nchunk = c->pair_chunks;
+        const cudaError_t e = launch_pair_f32(c->m.law, &p, c->pair_grid, c->st);
+        if (e != cudaSuccess) return e;
+        c->cur ^= 1;
+        c->step += 2;
+    }
+    return cudaSuccess;
+}
+
 // In the node form of F^b every ghost value depends only on its own boundary
 // node, so the step kernel writes the next step's ghosts itself (fused) and
 // the separate ghost kernel runs only when they are stale. The extrapolated
@@ -226,9 +265,8 @@ lbm_status do_step(lbm_ctx *c, int64_t nsteps)
     const bool prof = c->prof && (c->ev_step.size() < 200000);
     const bool fuse = c->cfg.fb_mode == LBM_FB_NODE;
     int64_t i = 0;
-    // a small lattice: up to MULTI_STEPS steps per launch (launches are
-    // counted and timed one step each when profiling)
-    if (c->multi_fn && !c->prof && nsteps > 1) {
+    // a small lattice: up to MULTI_STEPS steps per launch
+    if (c->multi_fn && grouped_steps(c, nsteps)) {
         if (c->ghosts_dirty) {
             CK(c, launch_ghosts(c->cfg.storage, edge_args(c, c->cur), c->edge_blk_end[3], c->st));
             c->ghosts_dirty = false;
@@ -240,6 +278,9 @@ lbm_status do_step(lbm_ctx *c, int64_t nsteps)
             c->step += len;
             i += len;
         }
+    } else if (grouped_steps(c, nsteps)) {
+        CK(c, do_pairs(c, nsteps / 2));
+        i = nsteps / 2 * 2;
     }
     for (; i < nsteps; ++i) {
         if (!fuse || c->ghosts_dirty) {
@@ -474,6 +515,46 @@ static void set_multi(lbm_ctx *c, int sms)
     c->multi_grid = (int)std::min<long long>((tasks + warps - 1) / warps, (long long)per_sm * sms);
 }
 
+// The two-step kernel (k_pair) takes the FP32 lattices that are too large for
+// k_multi. (16-bit storage would gain 1 to 5%: FP16 4096^2 314 -> 298 us a
+// step with a kernel of two nodes per lane, BF16 4096 x 2048 clamped 163.5 ->
+// 162.)
+static void set_pair(lbm_ctx *c, int sms)
+{
+    c->pair_grid = 0;
+    if (c->multi_fn || c->cfg.storage != STORE_F32 || c->cfg.fb_mode != LBM_FB_NODE || c->m.mufield) return;
+    if (c->L.nx < 8 || c->L.ny < 8) return;
+    if (dyn_env_choice() >= 0 || stripes_env_choice() >= 0 || step16_env_choice() >= 0) return;
+    const int per_sm = pair_blocks_f32(c->m.law);
+    if (per_sm < 1) return;
+    const int ny = c->L.ny, warps = 4 * per_sm * sms;
+    c->pair_strips = (c->L.nx + PAIR_COLUMNS - 1) / PAIR_COLUMNS;
+    // Rows per task, by a model of a launch's length in rows' time: a task
+    // takes one more row than it writes; the tasks come in rounds of one per
+    // warp, which even out once there are more than four; one long task per
+    // warp leaves the launch to its slowest warp; and the tasks of a
+    // non-periodic bottom or top row (traction Newton solves), which run
+    // first, take 11 rows longer. us per step, rows per task: 8192^2 1427
+    // with 16, 1406 with 32, 1661 with one task per warp; 4096 x 2048 clamped
+    // 201 with 12, 213 with 32, 300 with one task per warp; 2048 x 1024
+    // clamped 68 with 8, 83 with one task per warp; 1500 x 1000 periodic 67
+    // with 8, 49 with one task per warp.
+    double best = 0.0;
+    for (int h : {4, 6, 8, 12, 16, 24, 32, 0}) {
+        const int chunks = h ? (ny + h - 1) / h : std::min(warps / c->pair_strips, ny / 4);
+        if (chunks < 1) continue;
+        const double rows = (double)ny / chunks, rounds = (double)chunks * c->pair_strips / warps;
+        double t = (rounds > 4.0 ? rounds + 0.5 : std::ceil(rounds)) * (rows + 1.0);
+        if (rounds <= 1.0 && rows > 40.0) t *= 1.35;
+        if (!yper(c)) t = std::max(t, rows + 12.0);
+        if (best == 0.0 || t < best) {
+            best = t;
+            c->pair_chunks = chunks;
+        }
+    }
+    c->pair_grid = (int)std::min<long long>(((long long)c->pair_strips * c->pair_chunks + 3) / 4, (long long)per_sm * sms);
+}
+
 static lbm_status set_step_grid(lbm_ctx *c)
 {
     int sms = 0;
@@ -486,6 +567,7 @@ static lbm_status set_step_grid(lbm_ctx *c)
     if (g > needed) g = needed;
     c->grid_step = (int)(g < 1 ? 1 : g);
     set_multi(c, sms > 0 ? sms : 1);
+    set_pair(c, sms > 0 ? sms : 1);
     return LBM_OK;
 }
 
@@ -1086,9 +1168,9 @@ lbm_status lbm_step_async(lbm_ctx *c, int64_t nsteps)
 
 lbm_status lbm_step(lbm_ctx *c, int64_t nsteps)
 {
-    if (c && nsteps > 0) {
-        // the context's first synchronising step picks the step-launch
-        // variant for the lattice (tune_step)
+    if (c && nsteps > 0 && !grouped_steps(c, nsteps)) {
+        // the context's first synchronising call that takes its steps one
+        // to a launch picks the step-launch variant for the lattice (tune_step)
         lbm_status s = tlv::ctx_tune_steps(c);
         if (s != LBM_OK) return s;
     }

@@ -222,6 +222,19 @@ struct StepTimes {
     EdgeVal<R> val[MULTI_STEPS][4];
 };
 
+// Two steps in one pass (k_pair): a the step arguments of the second step
+// (a.fin the first's input, a.fout the second's output), g1 and v1 the edge
+// data of the first (as StepTimes' rows)
+constexpr int PAIR_SIDE_ROWS = 16;
+constexpr int PAIR_VEC = 4, PAIR_COLUMNS = 30 * PAIR_VEC;  // nodes per lane, columns per strip
+template <typename R>
+struct PairArgs {
+    StepArgs<R> a;
+    double g1[4];
+    EdgeVal<R> v1[4];
+    int nstrip, nchunk;  // strips of columns, chunks of rows
+};
+
 // A batch of lattices for one persistent launch
 constexpr int BATCH_MAX_MEMBERS = 4096;
 struct BatchList {

@@ -75,6 +75,7 @@ struct lbm_ctx {
     int grid_step = 1;
     const void *multi_fn = nullptr;  // many-steps kernel of a small lattice (set_multi), or nullptr
     int multi_block = 0, multi_grid = 0;
+    int pair_strips = 0, pair_chunks = 0, pair_grid = 0;  // two-step kernel (set_pair); 0 grid: not used
     int edge_blk_end[4] = {0, 0, 0, 0};
     std::string err;
     bool prof = false;
@@ -116,6 +117,12 @@ const void *multi_kernel_f64(int law);
 const void *multi_kernel_f32(int law);
 const void *multi_kernel_bf16(int law);
 const void *multi_kernel_f16(int law);
+
+// lbm_pair_f32.cu: two steps in one pass (PairArgs), the ghost columns it
+// reads with periodic x, resident blocks per SM
+cudaError_t launch_pair_f32(int law, const void *args, int grid, cudaStream_t st);
+cudaError_t launch_wide_f32(void *f, const Layout &L, cudaStream_t st);
+int pair_blocks_f32(int law);
 
 // lbm_aux.cu
 struct InitArgs {

@@ -493,7 +493,7 @@ __global__ void k_adj_inject(const InjectArgs<typename Prec<S>::R> a)
 // The cotangents of the finite-difference gradients of v0 go to ghat for the
 // transposed stencil of k_adj_init_fd.
 template <typename S>
-__global__ void __launch_bounds__(128) k_adj_init(const AdjInitArgs a)
+__global__ void __launch_bounds__(128) k_adj_init(const AdjInitArgs a, const InitConst<double> K)
 {
     using T = typename Prec<S>::R;
     const InitArgs &ia = a.ia;
@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(128) k_adj_init(const AdjInitArgs a)
         const int x = (int)(n % nx), y = (int)(n / nx);
         double f0[4][6];
         const LawP<double> mp = law_at(ia.m, n);
-        init_node(ia, x, y, mp, f0);
+        init_node(ia, K, x, y, mp, f0);
         double Un[6];
         for (int k = 0; k < 6; ++k) Un[k] = f0[0][k] + f0[1][k] + f0[2][k] + f0[3][k];
         Un[0] += 0.5 * dt * ia.b1;
@@ -545,8 +545,8 @@ __global__ void __launch_bounds__(128) k_adj_init(const AdjInitArgs a)
         double gm = -wi2c * (M[0] * Pm[0] + M[1] * Pm[1] + M[2] * Pm[2] + M[3] * Pm[3]);
         {
             double fR[4][6], fZ[4][6];
-            init_node(ia, x, y, unit, fR);
-            init_node(ia, x, y, LawP<double>{0.0, 0.0, 0.0, 0.0}, fZ);
+            init_node(ia, K, x, y, unit, fR);
+            init_node(ia, K, x, y, LawP<double>{0.0, 0.0, 0.0, 0.0}, fZ);
             for (int q = 0; q < 4; ++q)
                 for (int k = 0; k < 6; ++k) gm += h[q][k] * (fR[q][k] - fZ[q][k]);
         }
@@ -726,9 +726,9 @@ cudaError_t launch_adj_init(int storage, const AdjInitArgs &a, cudaStream_t st)
     const long long N = (long long)a.ia.L.nx * a.ia.L.ny;
     const int grid = grid_for(N, 128);
     if (storage == STORE_F64)
-        k_adj_init<double><<<grid, 128, 0, st>>>(a);
+        k_adj_init<double><<<grid, 128, 0, st>>>(a, init_const<double>(a.ia));
     else
-        k_adj_init<float><<<grid, 128, 0, st>>>(a);
+        k_adj_init<float><<<grid, 128, 0, st>>>(a, init_const<double>(a.ia));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_adj_init_fd<<<grid_for(N, 256), 256, 0, st>>>(a);

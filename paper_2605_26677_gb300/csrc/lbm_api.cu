@@ -310,9 +310,9 @@ lbm_status read_device(lbm_ctx *c, double *U, double *P, double *sigma, double *
     a.ustar = c->ustar;
     a.L = c->L;
     a.m = c->m;
-    a.dt = c->dt;
-    a.b1 = c->b[0];
-    a.b2 = c->b[1];
+    a.hdt = 0.5 * c->dt;
+    a.hb1 = 0.5 * c->dt * c->b[0];
+    a.hb2 = 0.5 * c->dt * c->b[1];
     a.U = U;
     a.P = P;
     a.sigma = sigma;
@@ -1254,10 +1254,9 @@ lbm_status lbm_diagnostics(lbm_ctx *c, double out[10])
     a.f = c->f[c->cur];
     a.L = c->L;
     a.m = c->m;
-    a.dt = c->dt;
     a.dx = c->cfg.dx;
-    a.b1 = c->b[0];
-    a.b2 = c->b[1];
+    a.hb1 = 0.5 * c->dt * c->b[0];
+    a.hb2 = 0.5 * c->dt * c->b[1];
     a.partial = c->d_diag;
     a.out = c->d_diag + (size_t)diag_blocks(c->L) * 10;
     CK(c, launch_diag(c->cfg.storage, a, c->st));

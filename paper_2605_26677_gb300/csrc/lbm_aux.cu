@@ -11,8 +11,15 @@ namespace tlv {
 
 // Initial populations (Sec. 3.4) followed by the collision of step 0, so the
 // stored state is f*^0; u* receives u0 - (dt/2) v0 + dt v^0 (Eq. 22).
+// FP32 and 16-bit storage: bound by latency at the 12 warps per SM that its
+// registers leave (4096 x 2048: 2.02 -> 1.81 ms with the constants from the
+// host; 1.17 ms at six blocks per SM, but with fewer registers the compiler
+// contracts its products differently and the start's last bits change). FP64
+// storage: bound by the FP64 pipe (11.9 -> 9.4 ms with one reciprocal for the
+// three tangent actions and Eq. (20) formed from them).
 template <typename T>
-__global__ void __launch_bounds__(128) k_init(const InitArgs a)
+__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 3)
+    k_init(const InitArgs a, const InitConst<typename std::conditional<sizeof(T) == 8, double, float>::type> K)
 {
     using R = typename std::conditional<sizeof(T) == 8, double, float>::type;  // compute type
     const int nx = a.L.nx, ny = a.L.ny;
@@ -23,22 +30,23 @@ __global__ void __launch_bounds__(128) k_init(const InitArgs a)
     const long long n1 = (long long)a.y1 * nx;
     for (long long n = (long long)a.y0 * nx + (long long)blockIdx.x * blockDim.x + threadIdx.x; n < n1;
          n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % nx), y = (int)(n / nx);
+        int x, y;
+        node_xy(n, nx, x, y);
         R f[4][6];  // f^0 - f_rest
         const LawP<R> m = law_cast<R>(law_at(a.m, n));
-        if (!init_node_ofs<R>(a, x, y, m, f)) atomicOr(a.status, ST_BAD_J);
+        if (!init_node_ofs<R>(a, K, x, y, m, f)) atomicOr(a.status, ST_BAD_J);
         // step-0 collision (Eqs. 10, 12, 14) on the offsets from the rest
         // state, which the collision leaves fixed
         R Un[6], dJ;
 #pragma unroll
         for (int k = 0; k < 6; ++k) Un[k] = (f[0][k] + f[2][k]) + (f[1][k] + f[3][k]);
-        Un[0] += (R)(0.5 * dt * a.b1);
-        Un[1] += (R)(0.5 * dt * a.b2);
+        Un[0] += K.hb1;
+        Un[1] += K.hb2;
         const R Gn[4] = {Un[2], Un[3], Un[4], Un[5]};
         R Pn[4], feq[4][6];
         piola_any_t<R>(a.m.law, Gn, m, Pn, dJ);
-        feq_ofs<R>(Un, Pn, c, feq);
-        const R src[2] = {(R)(dt * (2.0 - a.omega) * 0.125 * a.b1), (R)(dt * (2.0 - a.omega) * 0.125 * a.b2)};
+        feq_ofs<R>(Un, Pn, sizeof(R) == 8 ? K.r2c : R(2) / c, feq);
+        const R src[2] = {K.src1, K.src2};
 #pragma unroll
         for (int q = 0; q < 4; ++q)
 #pragma unroll
@@ -50,8 +58,15 @@ __global__ void __launch_bounds__(128) k_init(const InitArgs a)
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const double u0 = a.u0 ? a.u0[k * N + n] : 0.0;
-            a.ustar[k * a.L.uplane + (long long)y * a.L.upitch + x] =
-                (u0 - 0.5 * dt * a.U0[k * N + n]) + dt * (double)Un[k];
+            bool ok = true;
+            double v;
+            if constexpr (sizeof(R) == 8) {
+                v = Un[k];
+            } else {
+                v = widen_int(Un[k], ok);
+                if (!ok) v = (double)Un[k];
+            }
+            a.ustar[k * a.L.uplane + (long long)y * a.L.upitch + x] = (u0 - 0.5 * dt * a.U0[k * N + n]) + dt * v;
         }
     }
 }
@@ -67,9 +82,54 @@ __global__ void k_mu_plane(const double *mu, R *plane, Layout L)
     }
 }
 
+// Components [K0, K1) of sum_q f*_q at the node of b (its plane K0), in FP64
+// (offset form). A call of its own: as a branch the compiler would execute
+// its conversions beside the integer ones.
+template <typename T, int K0, int K1>
+__device__ __noinline__ void node_sums_cvt(const T *b, long long plane, double *S)
+{
+    for (int k = 0; k < K1 - K0; ++k) {
+        double s = 0.0;
+        for (int q = 0; q < 4; ++q) s += (double)ld_r(b[(q * 6 + k) * plane]);
+        S[k] = s;
+    }
+}
+
+// The same with the values widened on the integer pipe where they are normal
+template <typename T, int K0, int K1>
+__device__ __forceinline__ void node_sums(const T *f, const Layout &L, int x, int y, double *S)
+{
+    constexpr int n = K1 - K0;
+    const T *b = f + pidx(L, 0, K0, x, y);
+    T v[4][n];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int k = 0; k < n; ++k) v[q][k] = b[(q * 6 + k) * L.plane];
+    double d[4][n];
+    bool ok = true;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int k = 0; k < n; ++k) {
+            if constexpr (sizeof(T) == 8)
+                d[q][k] = v[q][k];
+            else
+                d[q][k] = widen_int(ld_r(v[q][k]), ok);
+        }
+#pragma unroll
+    for (int k = 0; k < n; ++k) S[k] = ((d[0][k] + d[1][k]) + d[2][k]) + d[3][k];
+    if constexpr (sizeof(T) < 8)
+        if (!ok) node_sums_cvt<T, K0, K1>(b, L.plane, S);
+}
+
 // U^n = sum_q f*_q - (dt/2) B, P(F^n), sigma = J^{-1} P F^T, u^n = u* - (dt/2) v^n
-// (the stored u* already holds u*^{n+1} = u*^n + dt v^n)
-template <typename T>
+// (the stored u* already holds u*^{n+1} = u*^n + dt v^n). Bound by the FP64
+// pipe: with the conversions off it, 18 sums and about 40 operations of the
+// stress per node are left (4096 x 2048 FP32: U and P 1.36 -> 0.88 ms,
+// u 0.33 -> 0.17 ms).
+// ST: U, P or sigma wanted, DISP: u.
+template <typename T, bool ST, bool DISP>
 __global__ void __launch_bounds__(128) k_read(const ReadArgs a)
 {
     const int nx = a.L.nx, ny = a.L.ny;
@@ -77,16 +137,14 @@ __global__ void __launch_bounds__(128) k_read(const ReadArgs a)
     const T *f = static_cast<const T *>(a.f);
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N;
          n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % nx), y = (int)(n / nx);
+        int x, y;
+        node_xy(n, nx, x, y);
         double S[6];
-        for (int k = 0; k < 6; ++k) {
-            double s = 0.0;
-            for (int q = 0; q < 4; ++q) s += (double)ld_r(f[pidx(a.L, q, k, x, y)]);
-            S[k] = s;
-        }
-        const double v1 = S[0] - 0.5 * a.dt * a.b1, v2 = S[1] - 0.5 * a.dt * a.b2;
+        if (DISP || a.U) node_sums<T, 0, 2>(f, a.L, x, y, S);
+        if (ST) node_sums<T, 2, 6>(f, a.L, x, y, S + 2);
+        const double v1 = S[0] - a.hb1, v2 = S[1] - a.hb2;
         const double G[4] = {S[2], S[3], S[4], S[5]};
-        if (a.U) {
+        if (ST && a.U) {
             a.U[0 * N + n] = v1;
             a.U[1 * N + n] = v2;
             a.U[2 * N + n] = 1.0 + G[0];
@@ -94,7 +152,7 @@ __global__ void __launch_bounds__(128) k_read(const ReadArgs a)
             a.U[4 * N + n] = G[2];
             a.U[5 * N + n] = 1.0 + G[3];
         }
-        if (a.P || a.sigma) {
+        if (ST && (a.P || a.sigma)) {
             double P[4], dJ;
             piola_any(a.m.law, G, law_at(a.m, n), P, dJ);
             if (a.P)
@@ -108,10 +166,10 @@ __global__ void __launch_bounds__(128) k_read(const ReadArgs a)
                 a.sigma[3 * N + n] = (P[2] * F[2] + P[3] * F[3]) / J;
             }
         }
-        if (a.u) {
+        if (DISP) {
             const long long ui = (long long)y * a.L.upitch + x;
-            a.u[0 * N + n] = a.ustar[ui] - 0.5 * a.dt * v1;
-            a.u[1 * N + n] = a.ustar[a.L.uplane + ui] - 0.5 * a.dt * v2;
+            a.u[0 * N + n] = a.ustar[ui] - a.hdt * v1;
+            a.u[1 * N + n] = a.ustar[a.L.uplane + ui] - a.hdt * v2;
         }
     }
 }
@@ -181,23 +239,22 @@ __global__ void __launch_bounds__(DIAG_THREADS) k_diag_partial(const DiagArgs a)
     r.gmax = 0.0;
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N;
          n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % nx), y = (int)(n / nx);
+        int x, y;
+        node_xy(n, nx, x, y);
         double S[6];
-        for (int k = 0; k < 6; ++k) {
-            double s = 0.0;
-            for (int q = 0; q < 4; ++q) s += (double)ld_r(f[pidx(a.L, q, k, x, y)]);
-            S[k] = s;
-        }
-        const double v1 = S[0] - 0.5 * a.dt * a.b1, v2 = S[1] - 0.5 * a.dt * a.b2;
+        node_sums<T, 0, 6>(f, a.L, x, y, S);
+        const double v1 = S[0] - a.hb1, v2 = S[1] - a.hb2;
         const double dJ = S[2] + S[5] + (S[2] * S[5] - S[3] * S[4]);
         r.s[0] += v1;
         r.s[1] += v2;
         for (int m = 0; m < 4; ++m) r.s[2 + m] += S[2 + m];
         r.s[6] += 0.5 * (v1 * v1 + v2 * v2) + energy_ofs(a.m.law, S[2], S[3], S[4], S[5], law_at(a.m, n));
-        r.jmin = fmin(r.jmin, 1.0 + dJ);
-        r.jmax = fmax(r.jmax, 1.0 + dJ);
-        r.gmax = fmax(r.gmax, sqrt(S[2] * S[2] + S[3] * S[3] + S[4] * S[4] + S[5] * S[5]));
+        const double J = 1.0 + dJ;
+        r.jmin = fmin(r.jmin, J);
+        r.jmax = fmax(r.jmax, J);
+        r.gmax = fmax(r.gmax, S[2] * S[2] + S[3] * S[3] + S[4] * S[4] + S[5] * S[5]);
     }
+    r.gmax = sqrt(r.gmax);  // the root of the largest square: the rounded root is monotone
     r = block_reduce(r);
     if (threadIdx.x == 0) {
         double *p = a.partial + (long long)blockIdx.x * 10;
@@ -256,7 +313,8 @@ cudaError_t launch_init(int storage, const InitArgs &a, cudaStream_t st)
     if (a.y1 == a.y0) return cudaSuccess;
     const int g = grid_for((long long)a.L.nx * (a.y1 - a.y0), 128);
     return with_storage(storage, [&](auto tag) {
-        k_init<decltype(tag)><<<g, 128, 0, st>>>(a);
+        using R = typename std::conditional<sizeof(tag) == 8, double, float>::type;
+        k_init<decltype(tag)><<<g, 128, 0, st>>>(a, init_const<R>(a));
         return cudaGetLastError();
     });
 }
@@ -265,7 +323,14 @@ cudaError_t launch_read(int storage, const ReadArgs &a, cudaStream_t st)
 {
     const int g = grid_for((long long)a.L.nx * a.L.ny, 128);
     return with_storage(storage, [&](auto tag) {
-        k_read<decltype(tag)><<<g, 128, 0, st>>>(a);
+        using T = decltype(tag);
+        const bool state = a.U || a.P || a.sigma;
+        if (state && a.u)
+            k_read<T, true, true><<<g, 128, 0, st>>>(a);
+        else if (state)
+            k_read<T, true, false><<<g, 128, 0, st>>>(a);
+        else
+            k_read<T, false, true><<<g, 128, 0, st>>>(a);
         return cudaGetLastError();
     });
 }

@@ -42,6 +42,18 @@ __device__ __forceinline__ float ld_r(float v) { return v; }
 __device__ __forceinline__ float ld_r(__half v) { return __half2float(v); }
 __device__ __forceinline__ float ld_r(__nv_bfloat16 v) { return __bfloat162float(v); }
 
+// A float as a double by the integer pipe, for zeros and normal floats; `ok`
+// becomes false for any other, and the caller then uses the conversion
+// instruction. That one occupies the FP64 pipe as long as an FP64
+// multiply-add does (64 cycles per warp), and on this GPU the FP64 pipe is
+// what bounds the read-out kernels.
+__device__ __forceinline__ double widen_int(float v, bool &ok)
+{
+    const unsigned b = __float_as_uint(v), t = b & 0x7fffffffu;
+    ok = ok && (t == 0u || t - 0x00800000u < 0x7f000000u);
+    const unsigned hi = (b & 0x80000000u) | ((t >> 3) + (t ? 0x38000000u : 0u));
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
 // round to the storage type (nearest even)
 template <typename S>
 __device__ __forceinline__ S to_store(double v);

@@ -5,7 +5,9 @@
 // less anyway, and whose every step computes in FP32).
 #pragma once
 #include "lbm_device.cuh"
+#include "lbm_edges.cuh"
 #include "lbm_internal.h"
+#include <type_traits>
 
 namespace tlv {
 
@@ -15,25 +17,35 @@ __device__ __forceinline__ long long pidx(const Layout &L, int q, int k, int x, 
 }
 
 
-// Second-order difference of a compact field along x (dir 0) or y (dir 1):
-// central inside, wrap-around when periodic, one-sided three-point stencil at
-// a non-periodic end (Sec. 3.4). h = 1 / (2 dx), computed once by the caller
-// (a multiply instead of an FP64 divide per difference).
-__device__ inline double fd(const double *a, int nx, int ny, int x, int y, int dir, int per, double h)
+// coordinates of node n (32-bit division where it suffices)
+__device__ __forceinline__ void node_xy(long long n, int nx, int &x, int &y)
+{
+    if (n >> 31) {
+        y = (int)(n / nx);
+    } else {
+        y = (int)((unsigned)n / (unsigned)nx);
+    }
+    x = (int)(n - (long long)y * nx);
+}
+
+// Second-order difference of a compact field along x (dir 0) or y (dir 1)
+// without its factor h = 1 / (2 dx): central inside, wrap-around when
+// periodic, one-sided three-point stencil at a non-periodic end (Sec. 3.4).
+__device__ __forceinline__ double fd(const double *a, int nx, int ny, int x, int y, int dir, int per)
 {
     const int n = dir == 0 ? nx : ny;
     const int i = dir == 0 ? x : y;
     auto at = [&](int j) { return dir == 0 ? a[(long long)y * nx + j] : a[(long long)j * nx + x]; };
-    if (per) return (at((i + 1) % n) - at((i - 1 + n) % n)) * h;
-    if (i == 0) return (-3.0 * at(0) + 4.0 * at(1) - at(2)) * h;
-    if (i == n - 1) return (3.0 * at(n - 1) - 4.0 * at(n - 2) + at(n - 3)) * h;
-    return (at(i + 1) - at(i - 1)) * h;
+    if (per) return at(i + 1 == n ? 0 : i + 1) - at(i == 0 ? n - 1 : i - 1);
+    if (i == 0) return -3.0 * at(0) + 4.0 * at(1) - at(2);
+    if (i == n - 1) return 3.0 * at(n - 1) - 4.0 * at(n - 2) + at(n - 3);
+    return at(i + 1) - at(i - 1);
 }
 
 // f^eq_q(U) - f^eq_q(U_rest) of Eq. (12): U_ofs = U - U_rest (v, F - I), P the
 // stress; f^eq is linear in U and in P, and P(I) = 0.
 template <typename R>
-__device__ __forceinline__ void feq_ofs(const R U[6], const R P[4], R c, R feq[4][6])
+__device__ __forceinline__ void feq_ofs(const R U[6], const R P[4], R r2c, R feq[4][6])
 {
     const R PhiX[6] = {-P[0], -P[2], -U[0], R(0), -U[1], R(0)};
     const R PhiY[6] = {-P[1], -P[3], R(0), -U[0], R(0), -U[1]};
@@ -41,7 +53,26 @@ __device__ __forceinline__ void feq_ofs(const R U[6], const R P[4], R c, R feq[4
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int k = 0; k < 6; ++k) feq[q][k] = R(0.25) * (U[k] + (R(2) / c) * (ci[q] * PhiX[k] + cj[q] * PhiY[k]));
+        for (int k = 0; k < 6; ++k) feq[q][k] = R(0.25) * (U[k] + r2c * (ci[q] * PhiX[k] + cj[q] * PhiY[k]));
+}
+
+// dP_i = C : dF_i for three directions at one F in FP64, the law chosen once
+// so that they share its reciprocal and cofactors
+__device__ __forceinline__ void tangent_jvp3(int law, const double G[4], const double d[3][4], const LawP<double> &m,
+                                             double dP[3][4])
+{
+    auto three = [&](auto L) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) jvp_ofs<decltype(L)::value, double>(G, d[i], m, dP[i]);
+    };
+    switch (law) {
+    case LAW_SVK: three(std::integral_constant<int, LAW_SVK>()); break;
+    case LAW_NH: three(std::integral_constant<int, LAW_NH>()); break;
+    case LAW_LOGNH: three(std::integral_constant<int, LAW_LOGNH>()); break;
+    case LAW_MR: three(std::integral_constant<int, LAW_MR>()); break;
+    case LAW_YEOH: three(std::integral_constant<int, LAW_YEOH>()); break;
+    default: three(std::integral_constant<int, LAW_GENT>()); break;
+    }
 }
 
 // f^0 - f_rest at node (x, y) in compute type R (f_rest = U_rest / 4: 1/4 in
@@ -49,12 +80,14 @@ __device__ __forceinline__ void feq_ofs(const R U[6], const R P[4], R c, R feq[4
 // correction -(dt/2) D_q f^eq of Eqs. (16)-(21), with the node's parameters.
 // Returns false if det F0 <= 0.
 template <typename R>
-__device__ inline bool init_node_ofs(const InitArgs &a, int x, int y, const LawP<R> &m, R f[4][6])
+__device__ inline bool init_node_ofs(const InitArgs &a, const InitConst<R> &K, int x, int y, const LawP<R> &m,
+                                     R f[4][6])
 {
     const int nx = a.L.nx, ny = a.L.ny;
     const long long N = (long long)nx * ny, n = (long long)y * nx + x;
     const int ci[4] = {1, 0, -1, 0}, cj[4] = {0, 1, 0, -1};
     const R c = (R)a.c, dt = (R)a.dt;
+    const R r2c = sizeof(R) == 8 ? K.r2c : R(2) / c;
     R U[6];  // U0 - U_rest
 #pragma unroll
     for (int k = 0; k < 6; ++k) U[k] = (R)(a.U0[k * N + n] - ((k == 2 || k == 5) ? 1.0 : 0.0));
@@ -62,18 +95,30 @@ __device__ inline bool init_node_ofs(const InitArgs &a, int x, int y, const LawP
     const R F[4] = {R(1) + U[2], U[3], U[4], R(1) + U[5]};
     R P[4], dJ;
     piola_any_t<R>(a.m.law, G, m, P, dJ);
-    feq_ofs<R>(U, P, c, f);
+    feq_ofs<R>(U, P, r2c, f);
     if (a.order == 2) {
         R gX[6], gY[6], dPX[4], dPY[4];
-        const double h = 0.5 / a.dx;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            gX[k] = (R)fd(a.U0 + k * N, nx, ny, x, y, 0, a.xper, h);
-            gY[k] = (R)fd(a.U0 + k * N, nx, ny, x, y, 1, a.yper, h);
+            gX[k] = (R)(fd(a.U0 + k * N, nx, ny, x, y, 0, a.xper) * K.h);
+            gY[k] = (R)(fd(a.U0 + k * N, nx, ny, x, y, 1, a.yper) * K.h);
         }
         // d_alpha P = C : d_alpha F (text after Eq. 18), as Jacobian actions (Eq. 8)
-        tangent_jvp_t<R>(a.m.law, F, gX + 2, m, dPX);
-        tangent_jvp_t<R>(a.m.law, F, gY + 2, m, dPY);
+        R dPt[4];  // FP64: C : d_t F too
+        if constexpr (sizeof(R) == 8) {
+            const R d[3][4] = {{gX[2], gX[3], gX[4], gX[5]}, {gY[2], gY[3], gY[4], gY[5]}, {gX[0], gY[0], gX[1], gY[1]}};
+            R o[3][4];
+            tangent_jvp3(a.m.law, G, d, m, o);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                dPX[k] = o[0][k];
+                dPY[k] = o[1][k];
+                dPt[k] = o[2][k];
+            }
+        } else {
+            tangent_jvp_t<R>(a.m.law, F, gX + 2, m, dPX);
+            tangent_jvp_t<R>(a.m.law, F, gY + 2, m, dPY);
+        }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const R i = (R)ci[q], j = (R)cj[q];
@@ -85,14 +130,20 @@ __device__ inline bool init_node_ofs(const InitArgs &a, int x, int y, const LawP
             Z[3] = gY[0] + c * i * gX[3] + c * j * gY[3];
             Z[4] = gX[1] + c * i * gX[4] + c * j * gY[4];
             Z[5] = gY[1] + c * i * gX[5] + c * j * gY[5];
-            tangent_jvp_t<R>(a.m.law, F, Z + 2, m, dP); // Eq. (20)
+            // Eq. (20); in FP64 from the actions at hand, C being linear
+            if constexpr (sizeof(R) == 8) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) dP[k] = dPt[k] + c * i * dPX[k] + c * j * dPY[k];
+            } else {
+                tangent_jvp_t<R>(a.m.law, F, Z + 2, m, dP);
+            }
             // Eq. (21): D_q f^eq = (f^eq)'(U0) Z_q, then Eq. (16)
-            const R Dq[6] = {R(0.25) * (Z[0] - (R(2) / c) * (i * dP[0] + j * dP[1])),
-                             R(0.25) * (Z[1] - (R(2) / c) * (i * dP[2] + j * dP[3])),
-                             R(0.25) * (Z[2] - (R(2) * i / c) * Z[0]),
-                             R(0.25) * (Z[3] - (R(2) * j / c) * Z[0]),
-                             R(0.25) * (Z[4] - (R(2) * i / c) * Z[1]),
-                             R(0.25) * (Z[5] - (R(2) * j / c) * Z[1])};
+            const R Dq[6] = {R(0.25) * (Z[0] - r2c * (i * dP[0] + j * dP[1])),
+                             R(0.25) * (Z[1] - r2c * (i * dP[2] + j * dP[3])),
+                             R(0.25) * (Z[2] - (r2c * i) * Z[0]),
+                             R(0.25) * (Z[3] - (r2c * j) * Z[0]),
+                             R(0.25) * (Z[4] - (r2c * i) * Z[1]),
+                             R(0.25) * (Z[5] - (r2c * j) * Z[1])};
 #pragma unroll
             for (int k = 0; k < 6; ++k) f[q][k] -= R(0.5) * dt * Dq[k];
         }
@@ -101,9 +152,10 @@ __device__ inline bool init_node_ofs(const InitArgs &a, int x, int y, const LawP
 }
 
 // f^0 at node (x, y) in full (not offset) form, FP64
-__device__ inline bool init_node(const InitArgs &a, int x, int y, const LawP<double> &m, double f[4][6])
+__device__ inline bool init_node(const InitArgs &a, const InitConst<double> &K, int x, int y, const LawP<double> &m,
+                                 double f[4][6])
 {
-    const bool ok = init_node_ofs<double>(a, x, y, m, f);
+    const bool ok = init_node_ofs<double>(a, K, x, y, m, f);
     for (int q = 0; q < 4; ++q) {
         f[q][2] += 0.25;
         f[q][5] += 0.25;

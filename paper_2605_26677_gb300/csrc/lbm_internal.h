@@ -138,6 +138,22 @@ struct InitArgs {
     int y0, y1;         // rows [y0, y1) written by this launch (its stencils read
                         // U0 one or two rows beyond them)
 };
+// What is the same for every node, formed once on the host: a thread that
+// forms it for its one node does so on the FP64 pipe
+template <typename R>
+struct InitConst {
+    R r2c;         // 2 / c (FP64 storage)
+    R hb1, hb2;    // (dt/2) b
+    R src1, src2;  // dt (2 - omega) b / 8
+    double h;      // 1 / (2 dx) of the differences
+};
+template <typename R>
+InitConst<R> init_const(const InitArgs &a)
+{
+    return InitConst<R>{R(2) / (R)a.c, (R)(0.5 * a.dt * a.b1), (R)(0.5 * a.dt * a.b2),
+                        (R)(a.dt * (2.0 - a.omega) * 0.125 * a.b1), (R)(a.dt * (2.0 - a.omega) * 0.125 * a.b2),
+                        0.5 / a.dx};
+}
 cudaError_t launch_init(int storage, const InitArgs &a, cudaStream_t st);
 // per-node mu (compact FP64) -> compute-type plane in the u* layout (zero padding)
 cudaError_t launch_mu_plane(int storage, const double *mu, void *plane, const Layout &L, cudaStream_t st);
@@ -149,7 +165,7 @@ struct ReadArgs {
     const double *ustar;
     Layout L;
     Material m;
-    double dt, b1, b2;
+    double hdt, hb1, hb2;  // dt / 2, (dt/2) b
     double *U;          // 6 x N or nullptr
     double *P;          // 4 x N or nullptr
     double *sigma;      // 4 x N or nullptr
@@ -161,7 +177,7 @@ struct DiagArgs {
     const void *f;
     Layout L;
     Material m;
-    double dt, dx, b1, b2;
+    double dx, hb1, hb2;  // hb = (dt/2) b
     double *partial;    // [blocks][10]
     double *out;        // [10]
 };

@@ -610,6 +610,7 @@ lbm_status backward_body(lbm_adjoint *a, double *g_mu_dev, double *g_v0_dev)
     ai.ghat = a->ghat;
     ai.tug = a->tug[cur];
     for (int e = 0; e < 4; ++e) ai.kind[e] = c->edge[e].kind;
+    ai.wi2c = c->cfg.omega * 0.5 / c->cfg.c;
     AK(a, launch_adj_init(c->cfg.storage, ai, c->st));
     AK(a, launch_plane_to_compact(a->gmu, g_mu_dev, c->L, c->st));
     AK(a, cudaEventRecord(a->ev[3], c->st));

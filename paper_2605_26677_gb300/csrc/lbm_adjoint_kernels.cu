@@ -488,8 +488,10 @@ __global__ void k_adj_inject(const InjectArgs<typename Prec<S>::R> a)
 
 // ---------------------------------------------------------------- init
 // Transpose of the step-0 collision and of f^0 = f^eq(U0) - (dt/2) D f^eq
-// (Eqs. 16-21) at each node, in FP64. f^0 is linear in v0 and affine in
-// (lambda, mu); its mu-derivative along lambda = r mu is f^0(r, 1) - f^0(0, 0).
+// (Eqs. 16-21) at each node, in FP64. f^0 is linear in v0 and affine in mu
+// (lambda = r mu): init_node_affine gives both parts at once. Bound by the
+// FP64 pipe (1024^2: 3.9 ms with f^0 evaluated for mu, 1 and 0 and a tangent
+// action per direction).
 // The cotangents of the finite-difference gradients of v0 go to ghat for the
 // transposed stencil of k_adj_init_fd.
 template <typename S>
@@ -502,19 +504,19 @@ __global__ void __launch_bounds__(128) k_adj_init(const AdjInitArgs a, const Ini
     const S *a0 = static_cast<const S *>(a.a0);
     const T *ubar = static_cast<const T *>(a.ubar);
     const int ci[4] = {1, 0, -1, 0}, cj[4] = {0, 1, 0, -1};
-    const double c = ia.c, dt = ia.dt, w = ia.omega, wi2c = w * 0.5 / c;
+    const double c = ia.c, dt = ia.dt, w = ia.omega, wi2c = a.wi2c;
+    const LawP<double> unit{ia.m.lam_ratio, 1.0, 0.0, 0.0};  // d(lambda, mu)/dmu
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N;
          n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % nx), y = (int)(n / nx);
-        double f0[4][6];
+        int x, y;
+        node_xy(n, nx, x, y);
         const LawP<double> mp = law_at(ia.m, n);
-        init_node(ia, K, x, y, mp, f0);
-        double Un[6];
-        for (int k = 0; k < 6; ++k) Un[k] = f0[0][k] + f0[1][k] + f0[2][k] + f0[3][k];
-        Un[0] += 0.5 * dt * ia.b1;
-        Un[1] += 0.5 * dt * ia.b2;
-        const double Fn[4] = {Un[2], Un[3], Un[4], Un[5]};
-        const double Gn[4] = {Un[2] - 1.0, Un[3], Un[4], Un[5] - 1.0};
+        double fz[4][6], fm[4][6];
+        init_node_affine(ia, K, x, y, unit, fz, fm);
+        double Gn[6];  // U - U_rest after the start
+        for (int k = 0; k < 6; ++k)
+            Gn[k] = ((fz[0][k] + fz[1][k]) + (fz[2][k] + fz[3][k])) + mp.mu * ((fm[0][k] + fm[1][k]) + (fm[2][k] + fm[3][k]));
+        const double Fn[4] = {1.0 + Gn[2], Gn[3], Gn[4], 1.0 + Gn[5]};
         const long long ui = (long long)y * ia.L.upitch + x;
         double h[4][6], Sa[6], bX[6], bY[6];
         for (int q = 0; q < 4; ++q)
@@ -532,9 +534,8 @@ __global__ void __launch_bounds__(128) k_adj_init(const AdjInitArgs a, const Ini
         const double ub[2] = {(double)ubar[ui], (double)ubar[ia.L.uplane + ui]};
         const double M[4] = {bX[0], bY[0], bX[1], bY[1]};
         double CM[4], Pm[4], dJ;
-        const LawP<double> unit{ia.m.lam_ratio, 1.0, 0.0, 0.0};  // d(lambda, mu)/dmu
         tangent_jvp(ia.m.law, Fn, M, mp, CM);
-        piola_any(ia.m.law, Gn, unit, Pm, dJ);
+        piola_any(ia.m.law, Gn + 2, unit, Pm, dJ);
         double g[6];
         g[0] = 0.25 * w * Sa[0] - wi2c * (bX[2] + bY[3]) + dt * ub[0];
         g[1] = 0.25 * w * Sa[1] - wi2c * (bX[4] + bY[5]) + dt * ub[1];
@@ -543,45 +544,41 @@ __global__ void __launch_bounds__(128) k_adj_init(const AdjInitArgs a, const Ini
             for (int k = 0; k < 6; ++k) h[q][k] = (1.0 - w) * h[q][k] + g[k];
         // mu: the step-0 collision and f^0 itself
         double gm = -wi2c * (M[0] * Pm[0] + M[1] * Pm[1] + M[2] * Pm[2] + M[3] * Pm[3]);
-        {
-            double fR[4][6], fZ[4][6];
-            init_node(ia, K, x, y, unit, fR);
-            init_node(ia, K, x, y, LawP<double>{0.0, 0.0, 0.0, 0.0}, fZ);
-            for (int q = 0; q < 4; ++q)
-                for (int k = 0; k < 6; ++k) gm += h[q][k] * (fR[q][k] - fZ[q][k]);
-        }
+        for (int q = 0; q < 4; ++q)
+            for (int k = 0; k < 6; ++k) gm += h[q][k] * fm[q][k];
         a.gmu[ui] += gm;
         // v0: f^eq(U0) at the node, and u*^0 = u0 - (dt/2) v0 + dt v^0
         double gv[2] = {-0.5 * dt * ub[0], -0.5 * dt * ub[1]};
         for (int q = 0; q < 4; ++q) {
-            gv[0] += 0.25 * (h[q][0] - (2.0 / c) * (ci[q] * h[q][2] + cj[q] * h[q][3]));
-            gv[1] += 0.25 * (h[q][1] - (2.0 / c) * (ci[q] * h[q][4] + cj[q] * h[q][5]));
+            gv[0] += 0.25 * (h[q][0] - K.r2c * (ci[q] * h[q][2] + cj[q] * h[q][3]));
+            gv[1] += 0.25 * (h[q][1] - K.r2c * (ci[q] * h[q][4] + cj[q] * h[q][5]));
         }
         a.gv0[n] = gv[0];
         a.gv0[N + n] = gv[1];
         // v0 through the gradients in D_q (order 2): Db_q = -(dt/2) h_q
         double gh[4] = {0.0, 0.0, 0.0, 0.0};  // d/d(dX v1, dX v2, dY v1, dY v2)
         if (ia.order == 2) {
-            double F0[4];
+            double F0[4], dPb[4] = {0.0, 0.0, 0.0, 0.0}, CdP[4];
             for (int m = 0; m < 4; ++m) F0[m] = ia.U0[(2 + m) * N + n];
             for (int q = 0; q < 4; ++q) {
-                const double i = ci[q], j = cj[q];
-                double Db[6], Zb[6], dPb[4], CdP[4];
-                for (int k = 0; k < 6; ++k) Db[k] = -0.5 * dt * h[q][k];
-                for (int k = 0; k < 6; ++k) Zb[k] = 0.25 * Db[k];
-                Zb[0] += -0.25 * (2.0 * i / c) * Db[2] - 0.25 * (2.0 * j / c) * Db[3];
-                Zb[1] += -0.25 * (2.0 * i / c) * Db[4] - 0.25 * (2.0 * j / c) * Db[5];
-                dPb[0] = -0.25 * (2.0 / c) * i * Db[0];
-                dPb[1] = -0.25 * (2.0 / c) * j * Db[0];
-                dPb[2] = -0.25 * (2.0 / c) * i * Db[1];
-                dPb[3] = -0.25 * (2.0 / c) * j * Db[1];
-                tangent_jvp(ia.m.law, F0, dPb, mp, CdP);  // C^T = C
-                for (int m = 0; m < 4; ++m) Zb[2 + m] += CdP[m];
-                gh[0] += c * i * Zb[0] + Zb[2];
-                gh[1] += c * i * Zb[1] + Zb[4];
-                gh[2] += c * j * Zb[0] + Zb[3];
-                gh[3] += c * j * Zb[1] + Zb[5];
+                const double i = ci[q], j = cj[q], s = -0.125 * dt;  // Db_q = -(dt/2) h_q
+                const double z0 = s * (h[q][0] - K.r2c * (i * h[q][2] + j * h[q][3]));
+                const double z1 = s * (h[q][1] - K.r2c * (i * h[q][4] + j * h[q][5]));
+                gh[0] += c * i * z0 + s * h[q][2];
+                gh[1] += c * i * z1 + s * h[q][4];
+                gh[2] += c * j * z0 + s * h[q][3];
+                gh[3] += c * j * z1 + s * h[q][5];
+                dPb[0] -= s * K.r2c * (i * h[q][0]);
+                dPb[1] -= s * K.r2c * (j * h[q][0]);
+                dPb[2] -= s * K.r2c * (i * h[q][1]);
+                dPb[3] -= s * K.r2c * (j * h[q][1]);
             }
+            // the tangent's part of every q at once, C being linear (C^T = C)
+            tangent_jvp(ia.m.law, F0, dPb, mp, CdP);
+            gh[0] += CdP[0];
+            gh[1] += CdP[2];
+            gh[2] += CdP[1];
+            gh[3] += CdP[3];
         }
         for (int m = 0; m < 4; ++m) a.ghat[m * N + n] = gh[m];
     }
@@ -589,7 +586,7 @@ __global__ void __launch_bounds__(128) k_adj_init(const AdjInitArgs a, const Ini
 
 // transpose of the second-order differences of Sec. 3.4 (central inside,
 // wrap-around when periodic, one-sided three-point stencils at the ends)
-__device__ __forceinline__ double fd_t(const double *g, int nx, int ny, int x, int y, int dir, int per, double dx)
+__device__ __forceinline__ double fd_t(const double *g, int nx, int ny, int x, int y, int dir, int per, double h)
 {
     const int n = dir == 0 ? nx : ny;
     const int i = dir == 0 ? x : y;
@@ -607,20 +604,21 @@ __device__ __forceinline__ double fd_t(const double *g, int nx, int ny, int x, i
         if (i == n - 2) s += -4.0 * at(n - 1);
         if (i == n - 3) s += 1.0 * at(n - 1);
     }
-    return s / (2.0 * dx);
+    return s * h;
 }
 
-__global__ void k_adj_init_fd(const AdjInitArgs a)
+__global__ void k_adj_init_fd(const AdjInitArgs a, double h)
 {
     const InitArgs &ia = a.ia;
     const int nx = ia.L.nx, ny = ia.L.ny;
     const long long N = (long long)nx * ny;
     for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N;
          n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % nx), y = (int)(n / nx);
+        int x, y;
+        node_xy(n, nx, x, y);
         for (int c = 0; c < 2; ++c)
-            a.gv0[c * N + n] += fd_t(a.ghat + c * N, nx, ny, x, y, 0, ia.xper, ia.dx) +
-                                fd_t(a.ghat + (2 + c) * N, nx, ny, x, y, 1, ia.yper, ia.dx);
+            a.gv0[c * N + n] += fd_t(a.ghat + c * N, nx, ny, x, y, 0, ia.xper, h) +
+                                fd_t(a.ghat + (2 + c) * N, nx, ny, x, y, 1, ia.yper, h);
     }
 }
 
@@ -731,7 +729,7 @@ cudaError_t launch_adj_init(int storage, const AdjInitArgs &a, cudaStream_t st)
         k_adj_init<float><<<grid, 128, 0, st>>>(a, init_const<double>(a.ia));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_adj_init_fd<<<grid_for(N, 256), 256, 0, st>>>(a);
+    k_adj_init_fd<<<grid_for(N, 256), 256, 0, st>>>(a, 0.5 / a.ia.dx);
     return cudaGetLastError();
 }
 

@@ -151,16 +151,66 @@ __device__ inline bool init_node_ofs(const InitArgs &a, const InitConst<R> &K, i
     return dJ > R(-1);
 }
 
-// f^0 at node (x, y) in full (not offset) form, FP64
-__device__ inline bool init_node(const InitArgs &a, const InitConst<double> &K, int x, int y, const LawP<double> &m,
-                                 double f[4][6])
+// f^0 - f_rest at node (x, y) in FP64 as fz + mu fm: for SVK, NH and log-NH
+// with lambda = r mu the stress and its tangent, and with them f^0, are linear
+// in mu (unit: the parameters at mu = 1). The terms of init_node_ofs, each
+// sorted into the part without P and the part with it.
+__device__ __forceinline__ void init_node_affine(const InitArgs &a, const InitConst<double> &K, int x, int y,
+                                                 const LawP<double> &unit, double fz[4][6], double fm[4][6])
 {
-    const bool ok = init_node_ofs<double>(a, K, x, y, m, f);
+    const int nx = a.L.nx, ny = a.L.ny;
+    const long long N = (long long)nx * ny, n = (long long)y * nx + x;
+    const double c = a.c;
+    double U[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) U[k] = a.U0[k * N + n] - ((k == 2 || k == 5) ? 1.0 : 0.0);
+    const double G[4] = {U[2], U[3], U[4], U[5]};
+    double P[4], dJ;
+    piola_any(a.m.law, G, unit, P, dJ);
+#pragma unroll
     for (int q = 0; q < 4; ++q) {
-        f[q][2] += 0.25;
-        f[q][5] += 0.25;
+        const double s = (q < 2 ? 0.25 : -0.25) * K.r2c;  // of Phi_X (even q) or Phi_Y
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            fz[q][k] = 0.25 * U[k];
+            fm[q][k] = 0.0;
+        }
+        const int o = q & 1;
+        fz[q][2 + o] -= s * U[0];
+        fz[q][4 + o] -= s * U[1];
+        fm[q][0] = -s * P[o];
+        fm[q][1] = -s * P[2 + o];
     }
-    return ok;
+    if (a.order != 2) return;
+    double gX[6], gY[6], dP[3][4];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        gX[k] = fd(a.U0 + k * N, nx, ny, x, y, 0, a.xper) * K.h;
+        gY[k] = fd(a.U0 + k * N, nx, ny, x, y, 1, a.yper) * K.h;
+    }
+    const double d[3][4] = {{gX[2], gX[3], gX[4], gX[5]}, {gY[2], gY[3], gY[4], gY[5]}, {gX[0], gY[0], gX[1], gY[1]}};
+    tangent_jvp3(a.m.law, G, d, unit, dP);
+    const double zb0 = dP[0][0] + dP[1][1], zb1 = dP[0][2] + dP[1][3];
+    const double dt8 = 0.125 * a.dt;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int o = q & 1;
+        const double sg = q < 2 ? 1.0 : -1.0, ci = sg * c, r = sg * K.r2c;
+        const double *g = o ? gY : gX;  // the difference along the direction
+        const double za0 = a.b1 + ci * g[0], za1 = a.b2 + ci * g[1];
+        const double Z[4] = {gX[0] + ci * g[2], gY[0] + ci * g[3], gX[1] + ci * g[4], gY[1] + ci * g[5]};
+        fz[q][0] -= dt8 * za0;
+        fz[q][1] -= dt8 * za1;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) fz[q][2 + k] -= dt8 * Z[k];
+        fz[q][2 + o] += dt8 * (r * za0);
+        fz[q][4 + o] += dt8 * (r * za1);
+        const double e0 = dP[2][o] + ci * dP[o][o], e1 = dP[2][2 + o] + ci * dP[o][2 + o];  // Eq. (20)
+        fm[q][0] -= dt8 * (zb0 - r * e0);
+        fm[q][1] -= dt8 * (zb1 - r * e1);
+        fm[q][2 + o] += dt8 * (r * zb0);
+        fm[q][4 + o] += dt8 * (r * zb1);
+    }
 }
 
 } // namespace tlv

@@ -233,6 +233,7 @@ struct AdjInitArgs {
     double *ghat;       // 4N compact scratch
     const void *tug;    // traction-edge cotangent of G for every q of a^0 (compute type, 4 planes)
     int kind[4];
+    double wi2c;        // omega / (2c)
 };
 cudaError_t launch_adj(int storage, int law, const void *args, int grid, cudaStream_t st);
 int adj_blocks_per_sm(int storage, int law);

@@ -247,6 +247,9 @@ cudaError_t do_pairs(lbm_ctx *c, int64_t pairs)
         p.a.ctr2 = c->d_ctr;
         p.nstrip = c->pair_strips;
         p.nchunk = c->pair_chunks;
+        p.nlong = c->pair_nlong;
+        p.hlong = c->pair_hlong;
+        p.hend = c->pair_hend;
         const cudaError_t e = launch_pair_f32(c->m.law, &p, c->pair_grid, c->st);
         if (e != cudaSuccess) return e;
         c->cur ^= 1;
@@ -529,29 +532,38 @@ static void set_pair(lbm_ctx *c, int sms)
     if (per_sm < 1) return;
     const int ny = c->L.ny, warps = 4 * per_sm * sms;
     c->pair_strips = (c->L.nx + PAIR_COLUMNS - 1) / PAIR_COLUMNS;
-    // Rows per task, by a model of a launch's length in rows' time: a task
-    // takes one more row than it writes; the tasks come in rounds of one per
-    // warp, which even out once there are more than four; one long task per
-    // warp leaves the launch to its slowest warp; and the tasks of a
-    // non-periodic bottom or top row (traction Newton solves), which run
-    // first, take 11 rows longer. us per step, rows per task: 8192^2 1427
-    // with 16, 1406 with 32, 1661 with one task per warp; 4096 x 2048 clamped
-    // 201 with 12, 213 with 32, 300 with one task per warp; 2048 x 1024
-    // clamped 68 with 8, 83 with one task per warp; 1500 x 1000 periodic 67
-    // with 8, 49 with one task per warp.
-    double best = 0.0;
-    for (int h : {4, 6, 8, 12, 16, 24, 32, 0}) {
-        const int chunks = h ? (ny + h - 1) / h : std::min(warps / c->pair_strips, ny / 4);
-        if (chunks < 1) continue;
-        const double rows = (double)ny / chunks, rounds = (double)chunks * c->pair_strips / warps;
-        double t = (rounds > 4.0 ? rounds + 0.5 : std::ceil(rounds)) * (rows + 1.0);
-        if (rounds <= 1.0 && rows > 40.0) t *= 1.35;
-        if (!yper(c)) t = std::max(t, rows + 12.0);
-        if (best == 0.0 || t < best) {
-            best = t;
-            c->pair_chunks = chunks;
+    // Rows per task. Where tasks of 16 rows come in more than three rounds of
+    // one per warp: 16, or 24 from 16 rounds on, and 6 for about the last
+    // two rounds, which leave the warps idle for less at the launch's end (us
+    // per step, 16 rows throughout / this: 4096 x 2048 clamped 194.5 / 187,
+    // 4096^2 377 / 370, 8192^2 1386 / 1366). Smaller lattices: by a model in
+    // rows' time, a task taking one more row than it writes, its rounds
+    // whole, one long task per warp leaving the launch to its slowest warp,
+    // and the tasks of a non-periodic bottom or top row (traction Newton
+    // solves), which run first, 11 rows longer (2048 x 1024 clamped 72 with 8
+    // rows, 79 with 16; 2048^2 109 with one task per warp, 119 with 16).
+    auto rounds_of = [&](int h) { return (double)((ny + h - 1) / h) * c->pair_strips / warps; };
+    c->pair_hend = 0;
+    if (rounds_of(16) > 3.0) {
+        c->pair_hlong = rounds_of(16) > 16.0 ? 24 : 16;
+        c->pair_hend = 6;
+    } else {
+        double best = 0.0;
+        for (int h : {4, 6, 8, 12, 16, std::max(4, (ny * c->pair_strips + warps - 1) / warps)}) {
+            const double rounds = rounds_of(h);
+            double t = std::ceil(rounds) * (h + 1.0);
+            if (rounds <= 1.0 && h > 40) t *= 1.35;
+            if (!yper(c)) t = std::max(t, h + 12.0);
+            if (best == 0.0 || t < best) {
+                best = t;
+                c->pair_hlong = h;
+            }
         }
     }
+    const int hl = c->pair_hlong, he = c->pair_hend;
+    const int tail = he ? std::min(ny, (int)((hl == 16 ? 2.0 : 1.5) * warps / c->pair_strips * he)) : 0;
+    c->pair_nlong = he ? (ny - tail) / hl : (ny + hl - 1) / hl;
+    c->pair_chunks = c->pair_nlong + (he ? (ny - c->pair_nlong * hl + he - 1) / he : 0);
     c->pair_grid = (int)std::min<long long>(((long long)c->pair_strips * c->pair_chunks + 3) / 4, (long long)per_sm * sms);
 }
 

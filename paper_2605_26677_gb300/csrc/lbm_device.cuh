@@ -244,7 +244,8 @@ struct PairArgs {
     StepArgs<R> a;
     double g1[4];
     EdgeVal<R> v1[4];
-    int nstrip, nchunk;  // strips of columns, chunks of rows
+    int nstrip, nchunk;      // strips of columns, chunks of rows
+    int nlong, hlong, hend;  // nlong chunks of hlong rows, the rest of hend
 };
 
 // A batch of lattices for one persistent launch

@@ -75,7 +75,8 @@ struct lbm_ctx {
     int grid_step = 1;
     const void *multi_fn = nullptr;  // many-steps kernel of a small lattice (set_multi), or nullptr
     int multi_block = 0, multi_grid = 0;
-    int pair_strips = 0, pair_chunks = 0, pair_grid = 0;  // two-step kernel (set_pair); 0 grid: not used
+    int pair_grid = 0;               // two-step kernel (set_pair); 0: not used
+    int pair_strips = 0, pair_chunks = 0, pair_nlong = 0, pair_hlong = 0, pair_hend = 0;  // as in PairArgs
     int edge_blk_end[4] = {0, 0, 0, 0};
     std::string err;
     bool prof = false;

@@ -182,7 +182,9 @@ __device__ __forceinline__ void pair_task(const PairArgs<S> &p, int chunk, int s
     const long long plane = a.L.plane;
     const S *__restrict__ fin = static_cast<const S *>(a.fin);
     S *__restrict__ fout = static_cast<S *>(a.fout);
-    const int ya = (int)((long long)ny * chunk / p.nchunk), yb = (int)((long long)ny * (chunk + 1) / p.nchunk);
+    const int over = max(chunk - p.nlong, 0);  // chunks of the short kind before this one
+    const int ya = (chunk - over) * p.hlong + over * p.hend;
+    const int yb = min(ny, ya + (chunk < p.nlong ? p.hlong : p.hend));
     const int c = (30 * strip + lane - 1) * VEC;
     const bool xper = a.kind[EDGE_LEFT] == BC_PERIODIC, yper = a.kind[EDGE_BOTTOM] == BC_PERIODIC;
     const bool ld = c <= (xper ? nx + 1 : nx);  // the lane's vector holds a column that some output needs
@@ -382,7 +384,7 @@ __device__ __forceinline__ void pair_task(const PairArgs<S> &p, int chunk, int s
 // velocities widened on the FP64 pipe 1580). Barriers that keep the warps of
 // a block on the same row made it slower (1756). The same bits as two
 // launches of k_step; us per step, k_step / k_pair: 8192^2 periodic 2145 /
-// 1401, 4096 x 2048 clamped 278 / 212, 2048^2 periodic 144 / 110. What binds it now
+// 1366, 4096 x 2048 clamped 278 / 187, 2048^2 periodic 144 / 109. What binds it now
 // is the latency of a warp's own chain at eight warps per SM (32% of issue
 // slots) and HBM at 5.3 TB/s; with the collisions taken out it moves its
 // data at 5.7 TB/s.
@@ -394,7 +396,10 @@ __global__ void __launch_bounds__(128, PAIR_BLOCKS) k_pair(const __grid_constant
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     PairSmem<S, VEC> *sm = reinterpret_cast<PairSmem<S, VEC> *>(smem) + wid;
     unsigned flags = 0;
-    dyn_tasks<DYN_STRIPES>(p.a.ctr, p.a.ctr_next, p.nstrip * p.nchunk, lane, [&](int task) {
+    // one counter: the tasks are few, and only a common order puts the long
+    // ones before the short ones (over four stripes 8192^2 took 1425 instead
+    // of 1386 us a step, 4096 x 2048 clamped 200 instead of 194)
+    dyn_tasks<1>(p.a.ctr, p.a.ctr_next, p.nstrip * p.nchunk, lane, [&](int task) {
         __syncwarp();
         // the chunks of the bottom and top rows, whose edge rules take longest, first
         const int i = task / p.nstrip;

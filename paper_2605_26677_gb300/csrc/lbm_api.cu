@@ -197,11 +197,34 @@ lbm_status record(lbm_ctx *c, std::vector<cudaEvent_t> &v)
     return LBM_OK;
 }
 
+// Whether k_multi takes the steps. Not with FP64 storage on a long lattice
+// whose rows mostly hold a node of a non-periodic side edge: k_multi applies
+// that edge's rule in the node's own warp, the FP64 step kernel 32 of them at
+// a time from a queue, which pays once warps take several rows each (26 x
+// 5535, traction: 157 us a step there, 165 with k_multi).
+bool use_multi(const lbm_ctx *c)
+{
+    if (!c->multi_fn) return false;
+    if (c->cfg.storage != STORE_F64 || xper(c)) return true;
+    const long long edge_tasks = (long long)c->L.ny * std::min(2, (c->L.nx + 31) / 32);
+    return edge_tasks <= (long long)c->multi_grid * (c->multi_block / 32);
+}
+
+// Whether k_pair takes the steps. Not where most of its tasks are those of
+// bottom and top edge rows (200000 x 8, traction: 87 us a step with it, 71
+// without; 40000 x 27: 45.3, 46.3), nor on a narrow lattice periodic in x,
+// whose wrapped columns every task copies (60 x 30000: 127, 120; 130 x 9000:
+// 60, 71).
+bool use_pair(const lbm_ctx *c)
+{
+    return c->pair_grid && (yper(c) || c->L.ny >= 24) && (!xper(c) || c->L.nx >= 100);
+}
+
 // Whether nsteps steps go several to a launch (k_multi, k_pair). Launches are
 // counted and timed one step each when profiling.
 bool grouped_steps(const lbm_ctx *c, int64_t nsteps)
 {
-    return (c->multi_fn || c->pair_grid) && !c->prof && nsteps > 1;
+    return (use_multi(c) || use_pair(c)) && !c->prof && nsteps > 1;
 }
 
 // `len` steps from a (a.fin and a.fout the two buffers) in one cooperative
@@ -269,7 +292,7 @@ lbm_status do_step(lbm_ctx *c, int64_t nsteps)
     const bool fuse = c->cfg.fb_mode == LBM_FB_NODE;
     int64_t i = 0;
     // a small lattice: up to MULTI_STEPS steps per launch
-    if (c->multi_fn && grouped_steps(c, nsteps)) {
+    if (use_multi(c) && grouped_steps(c, nsteps)) {
         if (c->ghosts_dirty) {
             CK(c, launch_ghosts(c->cfg.storage, edge_args(c, c->cur), c->edge_blk_end[3], c->st));
             c->ghosts_dirty = false;

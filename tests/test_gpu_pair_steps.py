@@ -11,7 +11,8 @@ from tests.test_gpu_multi_steps import compare, lbm  # noqa: F401
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("nx,ny,edges", [(8, 140000, "vttt"), (140000, 8, "vttt"), (9, 120001, "pppp"),
+@pytest.mark.parametrize("nx,ny,edges", [(8, 140000, "vttt"), (45000, 24, "vttt"), (140000, 8, "vvpp"),
+                                         (101, 11001, "pppp"),
                                          (119, 9001, "ppvt"), (120, 9001, "tvpp"), (121, 9001, "vttt"),
                                          (122, 9001, "pppp"), (1199, 1001, "pppp"), (1200, 999, "vtpp"),
                                          (1201, 1001, "tttv"), (1322, 1000, "ppvt")])

@@ -208,7 +208,8 @@ lbm_status lbm_init_device(lbm_ctx *ctx, const double *U0_dev, const double *u0_
  * steps of a small lattice (uniform material, node form of F^b) go in
  * cooperative launches of up to 64 steps each, those of a larger FP32 lattice
  * in launches of two steps, with the same results; such calls need no
- * variant and leave the choice to a later one.
+ * variant and leave the choice to a later one. While the context's stream is
+ * being captured every step is a launch of its own.
  * LBM_STEP16=regs or staged, LBM_DYN=0 or 1 and LBM_DYN_STRIPES=1 or 4 in the
  * environment restrict the choice (and keep one launch per step). */
 lbm_status lbm_step(lbm_ctx *ctx, int64_t nsteps);

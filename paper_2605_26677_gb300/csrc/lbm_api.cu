@@ -221,10 +221,18 @@ bool use_pair(const lbm_ctx *c)
 }
 
 // Whether nsteps steps go several to a launch (k_multi, k_pair). Launches are
-// counted and timed one step each when profiling.
+// counted and timed one step each when profiling; and while the stream is
+// being captured, so that a graph of an even number of steps leaves the state
+// in the buffer it was read from and can be replayed.
 bool grouped_steps(const lbm_ctx *c, int64_t nsteps)
 {
-    return (use_multi(c) || use_pair(c)) && !c->prof && nsteps > 1;
+    if (nsteps < 2 || c->prof || !(use_multi(c) || use_pair(c))) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->st, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cap == cudaStreamCaptureStatusNone;
 }
 
 // `len` steps from a (a.fin and a.fout the two buffers) in one cooperative
@@ -292,7 +300,8 @@ lbm_status do_step(lbm_ctx *c, int64_t nsteps)
     const bool fuse = c->cfg.fb_mode == LBM_FB_NODE;
     int64_t i = 0;
     // a small lattice: up to MULTI_STEPS steps per launch
-    if (use_multi(c) && grouped_steps(c, nsteps)) {
+    const bool grouped = grouped_steps(c, nsteps);
+    if (grouped && use_multi(c)) {
         if (c->ghosts_dirty) {
             CK(c, launch_ghosts(c->cfg.storage, edge_args(c, c->cur), c->edge_blk_end[3], c->st));
             c->ghosts_dirty = false;
@@ -304,7 +313,7 @@ lbm_status do_step(lbm_ctx *c, int64_t nsteps)
             c->step += len;
             i += len;
         }
-    } else if (grouped_steps(c, nsteps)) {
+    } else if (grouped) {
         CK(c, do_pairs(c, nsteps / 2));
         i = nsteps / 2 * 2;
     }

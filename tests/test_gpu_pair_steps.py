@@ -45,3 +45,34 @@ def test_asynchronous_steps_and_checkpoint(lbm):  # noqa: F811
         res.append(lbm.lbm_read_state(L.ctx)[0].view(np.uint64))
         L.close()
     assert np.array_equal(*res)
+
+
+@pytest.mark.parametrize("nx,ny,storage", [(96, 80, 0), (1300, 900, 1)])
+def test_captured_steps_can_be_replayed(lbm, nx, ny, storage):  # noqa: F811
+    """A graph of two steps replayed three times makes six steps."""
+    import torch
+
+    U0 = np.zeros((6, ny, nx))
+    U0[2] = U0[5] = 1.0
+    U0[0] = 0.02 * np.sin(2 * np.pi * np.arange(nx) / nx)[None, :]
+    res = []
+    for graph in (False, True):
+        s = torch.cuda.Stream()
+        L = lbm.Lattice(nx, ny, c=6.0, omega=1.9, storage=storage, stream=s)
+        lbm.lbm_set_material(L.ctx, 1, [1.5, 0.75])
+        lbm.lbm_init(L.ctx, U0)
+        lbm.lbm_step_async(L.ctx, 1)
+        lbm.lbm_sync(L.ctx)
+        if graph:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=s):
+                lbm.lbm_step_async(L.ctx, 2)
+            with torch.cuda.stream(s):
+                for _ in range(3):
+                    g.replay()
+        else:
+            lbm.lbm_step(L.ctx, 6)
+        lbm.lbm_sync(L.ctx)
+        res.append(lbm.lbm_read_state(L.ctx)[0].view(np.uint64))
+        L.close()
+    assert np.array_equal(*res)

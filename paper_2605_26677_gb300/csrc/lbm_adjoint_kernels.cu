@@ -489,9 +489,9 @@ __global__ void k_adj_inject(const InjectArgs<typename Prec<S>::R> a)
 // ---------------------------------------------------------------- init
 // Transpose of the step-0 collision and of f^0 = f^eq(U0) - (dt/2) D f^eq
 // (Eqs. 16-21) at each node, in FP64. f^0 is linear in v0 and affine in mu
-// (lambda = r mu): init_node_affine gives both parts at once. Bound by the
+// (lambda = r mu): init_node_parts gives both parts at once. Bound by the
 // FP64 pipe (1024^2: 3.9 ms with f^0 evaluated for mu, 1 and 0 and a tangent
-// action per direction).
+// action per direction, 0.7 now).
 // The cotangents of the finite-difference gradients of v0 go to ghat for the
 // transposed stencil of k_adj_init_fd.
 template <typename S>
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(128) k_adj_init(const AdjInitArgs a, const Ini
         node_xy(n, nx, x, y);
         const LawP<double> mp = law_at(ia.m, n);
         double fz[4][6], fm[4][6];
-        init_node_affine(ia, K, x, y, unit, fz, fm);
+        init_node_parts<true>(ia, K, x, y, unit, fz, fm);
         double Gn[6];  // U - U_rest after the start
         for (int k = 0; k < 6; ++k)
             Gn[k] = ((fz[0][k] + fz[1][k]) + (fz[2][k] + fz[3][k])) + mp.mu * ((fm[0][k] + fm[1][k]) + (fm[2][k] + fm[3][k]));

@@ -13,10 +13,11 @@ namespace tlv {
 // stored state is f*^0; u* receives u0 - (dt/2) v0 + dt v^0 (Eq. 22).
 // FP32 and 16-bit storage: bound by latency at the 12 warps per SM that its
 // registers leave (4096 x 2048: 2.02 -> 1.81 ms with the constants from the
-// host; 1.17 ms at six blocks per SM, but with fewer registers the compiler
+// host, 1.78 in blocks of two warps; 1.17 ms at six blocks per SM, but with fewer registers the compiler
 // contracts its products differently and the start's last bits change). FP64
 // storage: bound by the FP64 pipe (11.9 -> 9.4 ms with one reciprocal for the
-// three tangent actions and Eq. (20) formed from them).
+// three tangent actions and Eq. (20) formed from them, 7.2 without the
+// products with the directions' zeros).
 template <typename T>
 __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 3)
     k_init(const InitArgs a, const InitConst<typename std::conditional<sizeof(T) == 8, double, float>::type> K)
@@ -34,7 +35,12 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 3)
         node_xy(n, nx, x, y);
         R f[4][6];  // f^0 - f_rest
         const LawP<R> m = law_cast<R>(law_at(a.m, n));
-        if (!init_node_ofs<R>(a, K, x, y, m, f)) atomicOr(a.status, ST_BAD_J);
+        bool valid;
+        if constexpr (sizeof(R) == 8)
+            valid = init_node_parts<false>(a, K, x, y, m, f, f);
+        else
+            valid = init_node_ofs<R>(a, K, x, y, m, f);
+        if (!valid) atomicOr(a.status, ST_BAD_J);
         // step-0 collision (Eqs. 10, 12, 14) on the offsets from the rest
         // state, which the collision leaves fixed
         R Un[6], dJ;
@@ -45,7 +51,22 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 3)
         const R Gn[4] = {Un[2], Un[3], Un[4], Un[5]};
         R Pn[4], feq[4][6];
         piola_any_t<R>(a.m.law, Gn, m, Pn, dJ);
-        feq_ofs<R>(Un, Pn, sizeof(R) == 8 ? K.r2c : R(2) / c, feq);
+        if constexpr (sizeof(R) == 8) {
+            // feq_ofs without the products with the directions' zeros
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int o = q & 1;
+                const R s = (q < 2 ? R(0.25) : R(-0.25)) * K.r2c;
+#pragma unroll
+                for (int k = 0; k < 6; ++k) feq[q][k] = R(0.25) * Un[k];
+                feq[q][0] -= s * Pn[o];
+                feq[q][1] -= s * Pn[2 + o];
+                feq[q][2 + o] -= s * Un[0];
+                feq[q][4 + o] -= s * Un[1];
+            }
+        } else {
+            feq_ofs<R>(Un, Pn, R(2) / c, feq);
+        }
         const R src[2] = {K.src1, K.src2};
 #pragma unroll
         for (int q = 0; q < 4; ++q)

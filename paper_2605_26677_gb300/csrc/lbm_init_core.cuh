@@ -87,7 +87,7 @@ __device__ inline bool init_node_ofs(const InitArgs &a, const InitConst<R> &K, i
     const long long N = (long long)nx * ny, n = (long long)y * nx + x;
     const int ci[4] = {1, 0, -1, 0}, cj[4] = {0, 1, 0, -1};
     const R c = (R)a.c, dt = (R)a.dt;
-    const R r2c = sizeof(R) == 8 ? K.r2c : R(2) / c;
+    const R r2c = R(2) / c;
     R U[6];  // U0 - U_rest
 #pragma unroll
     for (int k = 0; k < 6; ++k) U[k] = (R)(a.U0[k * N + n] - ((k == 2 || k == 5) ? 1.0 : 0.0));
@@ -104,21 +104,8 @@ __device__ inline bool init_node_ofs(const InitArgs &a, const InitConst<R> &K, i
             gY[k] = (R)(fd(a.U0 + k * N, nx, ny, x, y, 1, a.yper) * K.h);
         }
         // d_alpha P = C : d_alpha F (text after Eq. 18), as Jacobian actions (Eq. 8)
-        R dPt[4];  // FP64: C : d_t F too
-        if constexpr (sizeof(R) == 8) {
-            const R d[3][4] = {{gX[2], gX[3], gX[4], gX[5]}, {gY[2], gY[3], gY[4], gY[5]}, {gX[0], gY[0], gX[1], gY[1]}};
-            R o[3][4];
-            tangent_jvp3(a.m.law, G, d, m, o);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                dPX[k] = o[0][k];
-                dPY[k] = o[1][k];
-                dPt[k] = o[2][k];
-            }
-        } else {
-            tangent_jvp_t<R>(a.m.law, F, gX + 2, m, dPX);
-            tangent_jvp_t<R>(a.m.law, F, gY + 2, m, dPY);
-        }
+        tangent_jvp_t<R>(a.m.law, F, gX + 2, m, dPX);
+        tangent_jvp_t<R>(a.m.law, F, gY + 2, m, dPY);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const R i = (R)ci[q], j = (R)cj[q];
@@ -130,13 +117,7 @@ __device__ inline bool init_node_ofs(const InitArgs &a, const InitConst<R> &K, i
             Z[3] = gY[0] + c * i * gX[3] + c * j * gY[3];
             Z[4] = gX[1] + c * i * gX[4] + c * j * gY[4];
             Z[5] = gY[1] + c * i * gX[5] + c * j * gY[5];
-            // Eq. (20); in FP64 from the actions at hand, C being linear
-            if constexpr (sizeof(R) == 8) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) dP[k] = dPt[k] + c * i * dPX[k] + c * j * dPY[k];
-            } else {
-                tangent_jvp_t<R>(a.m.law, F, Z + 2, m, dP);
-            }
+            tangent_jvp_t<R>(a.m.law, F, Z + 2, m, dP); // Eq. (20)
             // Eq. (21): D_q f^eq = (f^eq)'(U0) Z_q, then Eq. (16)
             const R Dq[6] = {R(0.25) * (Z[0] - r2c * (i * dP[0] + j * dP[1])),
                              R(0.25) * (Z[1] - r2c * (i * dP[2] + j * dP[3])),
@@ -151,12 +132,15 @@ __device__ inline bool init_node_ofs(const InitArgs &a, const InitConst<R> &K, i
     return dJ > R(-1);
 }
 
-// f^0 - f_rest at node (x, y) in FP64 as fz + mu fm: for SVK, NH and log-NH
-// with lambda = r mu the stress and its tangent, and with them f^0, are linear
-// in mu (unit: the parameters at mu = 1). The terms of init_node_ofs, each
-// sorted into the part without P and the part with it.
-__device__ __forceinline__ void init_node_affine(const InitArgs &a, const InitConst<double> &K, int x, int y,
-                                                 const LawP<double> &unit, double fz[4][6], double fm[4][6])
+// f^0 - f_rest at node (x, y) in FP64 with the node's parameters, its terms
+// added to fz (without P) and fm (with P), which may be one array: the terms
+// of init_node_ofs without the products with the directions' zeros. SPLIT: fm
+// starts from zero. For SVK, NH and log-NH with lambda = r mu the stress and its
+// tangent are linear in mu, and f^0 is fz + mu fm with fm that of mu = 1.
+// Returns false if det F0 <= 0.
+template <bool SPLIT>
+__device__ __forceinline__ bool init_node_parts(const InitArgs &a, const InitConst<double> &K, int x, int y,
+                                                const LawP<double> &m, double fz[4][6], double fm[4][6])
 {
     const int nx = a.L.nx, ny = a.L.ny;
     const long long N = (long long)nx * ny, n = (long long)y * nx + x;
@@ -166,22 +150,23 @@ __device__ __forceinline__ void init_node_affine(const InitArgs &a, const InitCo
     for (int k = 0; k < 6; ++k) U[k] = a.U0[k * N + n] - ((k == 2 || k == 5) ? 1.0 : 0.0);
     const double G[4] = {U[2], U[3], U[4], U[5]};
     double P[4], dJ;
-    piola_any(a.m.law, G, unit, P, dJ);
+    piola_any(a.m.law, G, m, P, dJ);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const double s = (q < 2 ? 0.25 : -0.25) * K.r2c;  // of Phi_X (even q) or Phi_Y
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             fz[q][k] = 0.25 * U[k];
-            fm[q][k] = 0.0;
+            if (SPLIT) fm[q][k] = 0.0;
         }
         const int o = q & 1;
         fz[q][2 + o] -= s * U[0];
         fz[q][4 + o] -= s * U[1];
-        fm[q][0] = -s * P[o];
-        fm[q][1] = -s * P[2 + o];
+        fm[q][0] -= s * P[o];
+        fm[q][1] -= s * P[2 + o];
     }
-    if (a.order != 2) return;
+    const bool ok = dJ > -1.0;
+    if (a.order != 2) return ok;
     double gX[6], gY[6], dP[3][4];
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
@@ -189,7 +174,7 @@ __device__ __forceinline__ void init_node_affine(const InitArgs &a, const InitCo
         gY[k] = fd(a.U0 + k * N, nx, ny, x, y, 1, a.yper) * K.h;
     }
     const double d[3][4] = {{gX[2], gX[3], gX[4], gX[5]}, {gY[2], gY[3], gY[4], gY[5]}, {gX[0], gY[0], gX[1], gY[1]}};
-    tangent_jvp3(a.m.law, G, d, unit, dP);
+    tangent_jvp3(a.m.law, G, d, m, dP);
     const double zb0 = dP[0][0] + dP[1][1], zb1 = dP[0][2] + dP[1][3];
     const double dt8 = 0.125 * a.dt;
 #pragma unroll
@@ -211,6 +196,7 @@ __device__ __forceinline__ void init_node_affine(const InitArgs &a, const InitCo
         fm[q][2 + o] += dt8 * (r * zb0);
         fm[q][4 + o] += dt8 * (r * zb1);
     }
+    return ok;
 }
 
 } // namespace tlv

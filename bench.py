@@ -172,13 +172,20 @@ def setup_ctx(lbm, w, storage, U0, u0):
     return L
 
 
-def timed_steps(lbm, torch, L, steps, warmup, dist, census_steps=10):
+def steps_per_launch(L, storage):
+    """Steps that one launch of the library takes in a long run: two on FP32
+    lattices of more than 2^20 nodes (k_pair, whose populations and u* move
+    once for both), one on the other lattices of this file."""
+    return 2 if storage == 1 and L.nx * L.ny > 1 << 20 else 1
+
+
+def timed_steps(lbm, torch, L, steps, warmup, dist, census_steps=10, storage=None):
     """Device time (ms) of exactly `steps` steps, CUDA events on the stream
     the kernels run on, with nothing else in the timed region. A short
-    untimed run with the library's per-launch events beforehand counts the
-    launches per step and splits a step between the bulk and the edge
-    kernel; the bulk kernel's average launch duration over the timed region
-    is then the region's time per step times its share."""
+    untimed run with the library's per-launch events beforehand (one launch
+    per step then) splits a step between the bulk and the edge kernel; the
+    bulk kernel's average time per step over the timed region is then the
+    region's time per step times its share."""
     st = torch.cuda.current_stream()
     lbm.lbm_step(L.ctx, warmup)
     lbm.lbm_profile(L.ctx, True)
@@ -201,7 +208,9 @@ def timed_steps(lbm, torch, L, steps, warmup, dist, census_steps=10):
     ms = e0.elapsed_time(e1)
     (ns, ts), (ne, te) = prof["step"], prof["edges"]
     share = ts / (ts + te) if ts + te > 0 else 1.0
-    info = {"launches_per_step": (ns + ne) / census_steps, "step_kernel_ms": ms / steps * share,
+    spl = steps_per_launch(L, storage)
+    info = {"launches_per_step": (ns + ne) / census_steps / spl, "steps_per_launch": spl,
+            "step_kernel_ms": ms / steps * share,
             "edge_kernel_ms": te / max(ne, 1), "step_variant": lbm.lbm_step_variant(L.ctx)}
     return ms, info
 
@@ -308,14 +317,16 @@ def run_ours(args, rank, ws, dist):
     N = wp.nx * wp.ny
     L = setup_ctx(lbm, wp, lbm.LBM_STORE_F32, Up, up)
     with ClockSampler(dev) as clk:
-        ms, tinfo = timed_steps(lbm, torch, L, args.steps, args.warmup, dist)
+        ms, tinfo = timed_steps(lbm, torch, L, args.steps, args.warmup, dist, storage=lbm.LBM_STORE_F32)
     clocks = clk.summary()
-    bpn = lbm.lbm_bytes_per_node_update(L.ctx)
+    bpn = lbm.lbm_bytes_per_node_update(L.ctx) / tinfo["steps_per_launch"]
     L.close()
     ms_max = max_over_ranks(ms, dist, "cuda")
     value = N * args.steps * ws / (ms_max * 1e-3) / 1e6
 
-    # roofline of the step kernel: its average launch duration over the timed region
+    # roofline of the step kernel: its average time per step over the timed
+    # region, against the bytes that a step moves (half of one single step's
+    # where a launch takes two)
     kern_ms = tinfo["step_kernel_ms"]
     achieved = bpn * N / (kern_ms * 1e-3) / 1e9
     traffic_bpn = recorded_traffic("fourier_periodic_%dx%d_f32" % (wp.nx, wp.ny))
@@ -341,8 +352,8 @@ def run_ours(args, rank, ws, dist):
         U0, u0 = w.fields()
         Nc = w.nx * w.ny
         L = setup_ctx(lbm, w, lbm.LBM_STORE_F32, U0, u0)
-        msc, ic = timed_steps(lbm, torch, L, k, 5, None)
-        bc = lbm.lbm_bytes_per_node_update(L.ctx)
+        msc, ic = timed_steps(lbm, torch, L, k, 5, None, storage=lbm.LBM_STORE_F32)
+        bc = lbm.lbm_bytes_per_node_update(L.ctx) / ic["steps_per_launch"]
         L.close()
         gbs = bc * Nc / (ic["step_kernel_ms"] * 1e-3) / 1e9
         tc = recorded_traffic("clamped_specimen_4096x2048_f32")
@@ -397,8 +408,10 @@ def run_ours(args, rank, ws, dist):
                      "frac": round(achieved / peak, 4), "peak_source": peak_kind,
                      "frac_of_nominal_7900": round(achieved / 7900.0, 4),
                      "traffic": None if traffic_bpn is None else traffic_bpn * N,
-                     "kernel": "k_step (fused pull-stream + collide + quadrature)",
-                     "bytes_per_node_update": bpn, "launch_ms": kern_ms, "step_variant": tinfo["step_variant"],
+                     "kernel": "k_pair (two fused pull-stream + collide + quadrature steps per pass)"
+                     if tinfo["steps_per_launch"] == 2 else "k_step (fused pull-stream + collide + quadrature)",
+                     "bytes_per_node_update": bpn, "steps_per_launch": tinfo["steps_per_launch"],
+                     "launch_ms": kern_ms * tinfo["steps_per_launch"], "step_variant": tinfo["step_variant"],
                      "edge_kernel_ms": tinfo["edge_kernel_ms"],
                      "launch_ms_source": "CUDA events around the timed region / launches (no per-launch events in it)"},
         "e2e": {"value": round(e2e, 1), "unit": UNIT, "h2d_bytes_per_step": h2d / args.steps,

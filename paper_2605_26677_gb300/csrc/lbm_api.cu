@@ -220,19 +220,39 @@ bool use_pair(const lbm_ctx *c)
     return c->pair_grid && (yper(c) || c->L.ny >= 24) && (!xper(c) || c->L.nx >= 100);
 }
 
+// Whether work enqueued on the context's stream is being captured (or the
+// stream cannot tell). From then on a graph may hold the address of the buffer
+// that the state lies in, and the counter set of a dynamic launch.
+bool capturing(lbm_ctx *c)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->st, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    if (cap == cudaStreamCaptureStatusNone) return false;
+    c->captured = true;
+    return true;
+}
+
+// Launches of two steps among nsteps. Each moves the state to the other
+// buffer, as one step does, so once work of the context has been captured they
+// come in twos: a call of an even number of steps then leaves the buffer and
+// the counters as a replayed graph expects them.
+int64_t pairs_of(const lbm_ctx *c, int64_t nsteps)
+{
+    if (!use_pair(c)) return 0;
+    return c->captured ? nsteps / 4 * 2 : nsteps / 2;
+}
+
 // Whether nsteps steps go several to a launch (k_multi, k_pair). Launches are
 // counted and timed one step each when profiling; and while the stream is
 // being captured, so that a graph of an even number of steps leaves the state
 // in the buffer it was read from and can be replayed.
-bool grouped_steps(const lbm_ctx *c, int64_t nsteps)
+bool grouped_steps(lbm_ctx *c, int64_t nsteps)
 {
-    if (nsteps < 2 || c->prof || !(use_multi(c) || use_pair(c))) return false;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->st, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return cap == cudaStreamCaptureStatusNone;
+    if (nsteps < 2 || c->prof || !(use_multi(c) || pairs_of(c, nsteps))) return false;
+    return !capturing(c);
 }
 
 // `len` steps from a (a.fin and a.fout the two buffers) in one cooperative
@@ -314,8 +334,9 @@ lbm_status do_step(lbm_ctx *c, int64_t nsteps)
             i += len;
         }
     } else if (grouped) {
-        CK(c, do_pairs(c, nsteps / 2));
-        i = nsteps / 2 * 2;
+        const int64_t pairs = pairs_of(c, nsteps);
+        CK(c, do_pairs(c, pairs));
+        i = 2 * pairs;
     }
     for (; i < nsteps; ++i) {
         if (!fuse || c->ghosts_dirty) {
@@ -403,6 +424,7 @@ lbm_status check_ready(lbm_ctx *c)
     if (!c) return fail(nullptr, LBM_ERR_ARG, "null context");
     if (!c->initialized) return fail(c, LBM_ERR_STATE, "lbm_init has not been called");
     CK(c, cudaSetDevice(c->cfg.device));
+    capturing(c);
     return LBM_OK;
 }
 
@@ -1196,6 +1218,7 @@ lbm_status lbm_init_device(lbm_ctx *c, const double *U0_dev, const double *u0_de
     lbm_status s = init_checks(c, U0_dev, order);
     if (s != LBM_OK) return s;
     CK(c, cudaSetDevice(c->cfg.device));
+    capturing(c);
     return init_common(c, U0_dev, u0_dev, order);
 }
 

@@ -64,6 +64,7 @@ struct lbm_ctx {
                                // counter stripes (chosen by the first lbm_step, or LBM_DYN)
     double *d_profile[4] = {nullptr, nullptr, nullptr, nullptr};
     int cur = 0;
+    bool captured = false;     // a graph may hold the buffers' addresses (capturing)
     long long step = 0;
     double dt = 0.0;
     tlv::Material m{};

@@ -21,6 +21,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include "lbm_ordered.cuh"
+
 namespace tlv {
 
 // ---------------------------------------------------------------- storage
@@ -317,10 +319,10 @@ template <typename R> __device__ __forceinline__ Dual<R> operator/(R a, Dual<R> 
     const R q = a / b.v;
     return {q, -q * b.d / b.v};
 }
-template <typename R> __device__ __forceinline__ Dual<R> log1p(Dual<R> a) { return {::log1p(a.v), a.d / (R(1) + a.v)}; }
+template <typename R> __device__ __forceinline__ Dual<R> log1p(Dual<R> a) { return {log1p(a.v), a.d / (R(1) + a.v)}; }
 template <typename R> __device__ __forceinline__ Dual<R> expm1(Dual<R> a)
 {
-    const R e = ::expm1(a.v);
+    const R e = expm1(a.v);
     return {e, (R(1) + e) * a.d};
 }
 
@@ -350,7 +352,7 @@ __device__ __forceinline__ void piola_inv(const V G[4], const LawP<R> &m, V P[4]
     if (LAW == LAW_MR)
         s1 = V(m.mu);
     else if (LAW == LAW_YEOH)
-        s1 = m.mu + (R(2) * m.p2) * A + (R(3) * m.p3) * (A * A);
+        s1 = m.mu + R(R(2) * m.p2) * A + R(R(3) * m.p3) * (A * A);
     else
         s1 = m.mu / (R(2) * (R(1) - A / V(m.p2)));
     const V c1 = R(2.0 / 3.0) * tc;

@@ -27,6 +27,11 @@ __device__ __forceinline__ double newton_tol<double>(double tmax, double, double
     return 1e-13 * (tmax > 1.0 ? tmax : 1.0);
 }
 template <>
+__device__ __forceinline__ Ordered newton_tol<Ordered>(Ordered tmax, Ordered, Ordered)
+{
+    return Ordered(newton_tol<double>(tmax.v, 0.0, 0.0));
+}
+template <>
 __device__ __forceinline__ float newton_tol<float>(float tmax, float mu, float gmax)
 {
     return 4e-6f * (tmax + mu * gmax) + 1e-30f;
@@ -147,14 +152,24 @@ __device__ bool traction_newton(int e, R G[4], const R Tb[2], const LawP<R> &m)
     return fmax(fabs(r[0]), fabs(r[1])) <= newton_tol<R>(tmax, mus, gmax);
 }
 
-// The Newton solve of a law with a logarithm in FP64, compiled on its own:
-// inlined, the compiler contracts its products differently from kernel to
-// kernel, and a run's last bit would depend on which kernel took its steps.
-template <int LAW, typename R>
-__device__ __noinline__ bool traction_newton_call(int e, R G[4], R T0, R T1, const LawP<R> &m)
+// The Newton solve of a law with a logarithm in FP64, with its roundings fixed
+// by the source (Ordered): contracted by the compiler, a run's last bit would
+// depend on which kernel took its steps. Inlined, because a call costs the
+// whole kernel its registers (us a step, called / inlined: 2744 x 2929 periodic
+// MR 3305 / 3060, Yeoh 2855 / 2587, Gent 3224 / 2789; with traction edges
+// 121 x 971 log-NH 136 / 95, MR 304 / 253). Left to the compiler's contraction
+// the solve itself is 1 to 2.5% faster (64^2 with traction edges, own
+// launches: MR 186.6 / 191.4, Yeoh 156.9 / 161.2, Gent 183.2 / 186.2).
+template <int LAW>
+__device__ __forceinline__ bool traction_newton_ordered(int e, double G[4], const double Tb[2], const LawP<double> &m)
 {
-    const R Tb[2] = {T0, T1};
-    return traction_newton<LAW, R>(e, G, Tb, m);
+    using R = Ordered;
+    R Go[4] = {R(G[0]), R(G[1]), R(G[2]), R(G[3])};
+    const R To[2] = {R(Tb[0]), R(Tb[1])};
+    const bool ok = traction_newton<LAW, R>(e, Go, To, LawP<R>{R(m.lam), R(m.mu), R(m.p2), R(m.p3)});
+#pragma unroll
+    for (int k = 0; k < 4; ++k) G[k] = Go[k].v;
+    return ok;
 }
 
 // Edge data of one boundary node at t^n + dt/2 in the compute type, and the
@@ -196,7 +211,7 @@ __device__ __forceinline__ void edge_ghost(int e, int kind, const R fo[6], const
         const R Tb[2] = {v0, v1};
         bool ok;
         if constexpr (sizeof(R) == 8 && LAW >= LAW_LOGNH)
-            ok = traction_newton_call<LAW, R>(e, G, v0, v1, m);
+            ok = traction_newton_ordered<LAW>(e, G, Tb, m);
         else
             ok = traction_newton<LAW, R>(e, G, Tb, m);
         if (!ok) flags |= ST_NEWTON;

@@ -5,6 +5,7 @@
 // a device step counter and a small diagnostics scratch area. Every device
 // operation is enqueued on the stream given at creation.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -256,7 +257,11 @@ bool grouped_steps(lbm_ctx *c, int64_t nsteps)
 }
 
 // `len` steps from a (a.fin and a.fout the two buffers) in one cooperative
-// launch; the edges' data of the steps go along as an argument
+// launch; the edges' data of the steps go along as an argument. A grid that
+// does not fit at once is refused (cudaErrorCooperativeLaunchTooLarge): it is
+// sized for the whole device, and a stream may have fewer SMs, or a limit may
+// have been set since. LBM_MULTI_REFUSE_TEST=n in the environment asks for one
+// in the n-th launch of the process.
 template <typename T>
 cudaError_t launch_multi(lbm_ctx *c, StepArgs<T> a, int len)
 {
@@ -269,9 +274,15 @@ cudaError_t launch_multi(lbm_ctx *c, StepArgs<T> a, int len)
     unsigned *count = c->d_ctr + 2 * DYN_SET_WORDS;
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned), c->st);
     if (e != cudaSuccess) return e;
+    static const int refuse = [] {
+        const char *v = std::getenv("LBM_MULTI_REFUSE_TEST");
+        return v ? std::atoi(v) : 0;
+    }();
+    static std::atomic<int> launches{0};
+    const int grid = refuse && ++launches == refuse ? 1 << 20 : c->multi_grid;
     void *params[] = {&a, &tab, &len, &count};
-    return cudaLaunchCooperativeKernel(c->multi_fn, dim3((unsigned)c->multi_grid), dim3((unsigned)c->multi_block),
-                                       params, 0, c->st);
+    return cudaLaunchCooperativeKernel(c->multi_fn, dim3((unsigned)grid), dim3((unsigned)c->multi_block), params, 0,
+                                       c->st);
 }
 
 // 2 `pairs` steps with the two-step kernel
@@ -328,7 +339,12 @@ lbm_status do_step(lbm_ctx *c, int64_t nsteps)
         }
         for (; nsteps - i > 1;) {
             const int len = (int)std::min<int64_t>(nsteps - i, MULTI_STEPS);
-            CK(c, launch_multi(c, step_args<T>(c, c->cur), len));
+            const cudaError_t e = launch_multi(c, step_args<T>(c, c->cur), len);
+            if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+                cudaGetLastError();  // clear it: the rest goes one step to a launch
+                break;
+            }
+            CK(c, e);
             c->cur ^= len & 1;
             c->step += len;
             i += len;

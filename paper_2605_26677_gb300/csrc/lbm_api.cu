@@ -256,12 +256,19 @@ bool grouped_steps(lbm_ctx *c, int64_t nsteps)
     return !capturing(c);
 }
 
+int env_int(const char *name)
+{
+    const char *v = std::getenv(name);
+    return v ? std::atoi(v) : 0;
+}
+
 // `len` steps from a (a.fin and a.fout the two buffers) in one cooperative
 // launch; the edges' data of the steps go along as an argument. A grid that
 // does not fit at once is refused (cudaErrorCooperativeLaunchTooLarge): it is
 // sized for the whole device, and a stream may have fewer SMs, or a limit may
 // have been set since. LBM_MULTI_REFUSE_TEST=n in the environment asks for one
-// in the n-th launch of the process.
+// in the n-th launch of the process, and LBM_MULTI_STALL_TEST=n starts the
+// barrier's count one too low in it, so that its first wait runs out.
 template <typename T>
 cudaError_t launch_multi(lbm_ctx *c, StepArgs<T> a, int len)
 {
@@ -271,15 +278,13 @@ cudaError_t launch_multi(lbm_ctx *c, StepArgs<T> a, int len)
             tab.g[k][e] = ctx_time_factor(c, e, c->step + k);
             tab.val[k][e] = edge_val<T>(c->edge[e].value, tab.g[k][e], a.c);
         }
-    unsigned *count = c->d_ctr + 2 * DYN_SET_WORDS;
-    cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned), c->st);
-    if (e != cudaSuccess) return e;
-    static const int refuse = [] {
-        const char *v = std::getenv("LBM_MULTI_REFUSE_TEST");
-        return v ? std::atoi(v) : 0;
-    }();
+    static const int refuse = env_int("LBM_MULTI_REFUSE_TEST"), stall = env_int("LBM_MULTI_STALL_TEST");
     static std::atomic<int> launches{0};
-    const int grid = refuse && ++launches == refuse ? 1 << 20 : c->multi_grid;
+    const int launch = refuse || stall ? ++launches : 0;
+    unsigned *count = c->d_ctr + 2 * DYN_SET_WORDS;
+    cudaError_t e = cudaMemsetAsync(count, stall && launch == stall ? 0xff : 0, sizeof(unsigned), c->st);
+    if (e != cudaSuccess) return e;
+    const int grid = refuse && launch == refuse ? 1 << 20 : c->multi_grid;
     void *params[] = {&a, &tab, &len, &count};
     return cudaLaunchCooperativeKernel(c->multi_fn, dim3((unsigned)grid), dim3((unsigned)c->multi_block), params, 0,
                                        c->st);

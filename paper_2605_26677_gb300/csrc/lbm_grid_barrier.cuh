@@ -5,12 +5,14 @@
 
 namespace tlv {
 
+constexpr unsigned long long BARRIER_LIMIT_NS = 1000000000ull;
+
 // Every block adds one to *count, which is zero when the launch begins, and
 // waits until it reaches `target` (blocks x barriers passed so far). Stores
 // made by any block before the barrier are visible after it to loads that go
 // past the L1 cache. The whole block calls it; false if the wait ran out
 // (the other blocks' waits then run out too, and every block returns).
-__device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, unsigned long long limit_ns = 1000000000ull)
+__device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target)
 {
     __syncthreads();
     int ok = 1;
@@ -25,7 +27,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, u
                 const unsigned long long t = global_ns();
                 if (t0 == 0) {
                     t0 = t;
-                } else if (t - t0 > limit_ns) {
+                } else if (t - t0 > BARRIER_LIMIT_NS) {
                     ok = 0;
                     break;
                 }

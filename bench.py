@@ -172,14 +172,7 @@ def setup_ctx(lbm, w, storage, U0, u0):
     return L
 
 
-def steps_per_launch(L, storage):
-    """Steps that one launch of the library takes in a long run: two on FP32
-    lattices of more than 2^20 nodes (k_pair, whose populations and u* move
-    once for both), one on the other lattices of this file."""
-    return 2 if storage == 1 and L.nx * L.ny > 1 << 20 else 1
-
-
-def timed_steps(lbm, torch, L, steps, warmup, dist, census_steps=10, storage=None):
+def timed_steps(lbm, torch, L, steps, warmup, dist, census_steps=10):
     """Device time (ms) of exactly `steps` steps, CUDA events on the stream
     the kernels run on, with nothing else in the timed region. A short
     untimed run with the library's per-launch events beforehand (one launch
@@ -208,10 +201,13 @@ def timed_steps(lbm, torch, L, steps, warmup, dist, census_steps=10, storage=Non
     ms = e0.elapsed_time(e1)
     (ns, ts), (ne, te) = prof["step"], prof["edges"]
     share = ts / (ts + te) if ts + te > 0 else 1.0
-    spl = steps_per_launch(L, storage)
-    info = {"launches_per_step": (ns + ne) / census_steps / spl, "steps_per_launch": spl,
-            "step_kernel_ms": ms / steps * share,
-            "edge_kernel_ms": te / max(ne, 1), "step_variant": lbm.lbm_step_variant(L.ctx)}
+    # steps per launch of the timed call; k_pair takes an odd last step as a launch of its own
+    spl = lbm.lbm_steps_per_launch(L.ctx, steps)
+    launches = -(-steps // spl) if spl != 2 else steps // 2 + steps % 2
+    info = {"launches_per_step": launches / steps + ne / census_steps, "steps_per_launch": spl,
+            "step_kernel_ms": ms / steps * share, "edge_kernel_ms": te / max(ne, 1),
+            # the variant of single-step launches, where the timed region had them
+            "step_variant": lbm.lbm_step_variant(L.ctx) if spl == 1 else None}
     return ms, info
 
 
@@ -317,9 +313,9 @@ def run_ours(args, rank, ws, dist):
     N = wp.nx * wp.ny
     L = setup_ctx(lbm, wp, lbm.LBM_STORE_F32, Up, up)
     with ClockSampler(dev) as clk:
-        ms, tinfo = timed_steps(lbm, torch, L, args.steps, args.warmup, dist, storage=lbm.LBM_STORE_F32)
+        ms, tinfo = timed_steps(lbm, torch, L, args.steps, args.warmup, dist)
     clocks = clk.summary()
-    bpn = lbm.lbm_bytes_per_node_update(L.ctx) / tinfo["steps_per_launch"]
+    bpn = lbm.lbm_bytes_per_node_update(L.ctx) / min(2, tinfo["steps_per_launch"])
     L.close()
     ms_max = max_over_ranks(ms, dist, "cuda")
     value = N * args.steps * ws / (ms_max * 1e-3) / 1e6
@@ -352,8 +348,8 @@ def run_ours(args, rank, ws, dist):
         U0, u0 = w.fields()
         Nc = w.nx * w.ny
         L = setup_ctx(lbm, w, lbm.LBM_STORE_F32, U0, u0)
-        msc, ic = timed_steps(lbm, torch, L, k, 5, None, storage=lbm.LBM_STORE_F32)
-        bc = lbm.lbm_bytes_per_node_update(L.ctx) / ic["steps_per_launch"]
+        msc, ic = timed_steps(lbm, torch, L, k, 5, None)
+        bc = lbm.lbm_bytes_per_node_update(L.ctx) / min(2, ic["steps_per_launch"])
         L.close()
         gbs = bc * Nc / (ic["step_kernel_ms"] * 1e-3) / 1e9
         tc = recorded_traffic("clamped_specimen_4096x2048_f32")
@@ -409,7 +405,8 @@ def run_ours(args, rank, ws, dist):
                      "frac_of_nominal_7900": round(achieved / 7900.0, 4),
                      "traffic": None if traffic_bpn is None else traffic_bpn * N,
                      "kernel": "k_pair (two fused pull-stream + collide + quadrature steps per pass)"
-                     if tinfo["steps_per_launch"] == 2 else "k_step (fused pull-stream + collide + quadrature)",
+                     if tinfo["steps_per_launch"] == 2 else "k_step (fused pull-stream + collide + quadrature)"
+                     if tinfo["steps_per_launch"] == 1 else "k_multi (many steps per launch)",
                      "bytes_per_node_update": bpn, "steps_per_launch": tinfo["steps_per_launch"],
                      "launch_ms": kern_ms * tinfo["steps_per_launch"], "step_variant": tinfo["step_variant"],
                      "edge_kernel_ms": tinfo["edge_kernel_ms"],

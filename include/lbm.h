@@ -222,7 +222,15 @@ lbm_status lbm_step(lbm_ctx *ctx, int64_t nsteps);
 /* As lbm_step without waiting; check later with lbm_sync. */
 lbm_status lbm_step_async(lbm_ctx *ctx, int64_t nsteps);
 
-/* The step-launch variant the context runs now (host outputs, either may be
+/* Steps per launch of a call of nsteps >= 1 as the context stands (host
+ * output): up to 64 (a small lattice), 2, or 1 (the launches that
+ * lbm_step_variant describes). A last launch may take fewer, and an odd step
+ * is a launch of its own. 1 while lbm_profile records or the stream is being
+ * captured. No device work. */
+lbm_status lbm_steps_per_launch(lbm_ctx *ctx, int64_t nsteps, int32_t *steps);
+
+/* The step-launch variant the context runs now where a launch takes one step
+ * (lbm_steps_per_launch; host outputs, either may be
  * NULL): *staged = 1 for the shared-memory staged 16-bit kernel, 0 for the
  * register kernel; *dynamic = 0 for static task order, else the number of
  * device counters the dynamic claims are spread over (1 or 4; 1 only for the
@@ -260,7 +268,10 @@ lbm_status lbm_load(lbm_ctx *ctx, const void *buf, size_t bytes);
 lbm_status lbm_info(lbm_ctx *ctx, int64_t *step, double *t, double *dt);
 
 /* Per-kernel timing with CUDA events on the context's stream. enable != 0
- * starts recording (and clears earlier records), 0 stops. lbm_profile_read
+ * starts recording (and clears earlier records), 0 stops. While it records
+ * every step is a launch of its own, also where a launch takes several steps
+ * otherwise (lbm_steps_per_launch): it then times another kernel than such a
+ * run launches, and a slower one. lbm_profile_read
  * synchronises and returns, for each of the kernels below, the number of
  * timed launches and their total device time in milliseconds:
  *   out[0], out[1]: fused collide-stream kernel (launches, ms)
@@ -268,9 +279,10 @@ lbm_status lbm_info(lbm_ctx *ctx, int64_t *step, double *t, double *dt);
 lbm_status lbm_profile(lbm_ctx *ctx, int32_t enable);
 lbm_status lbm_profile_read(lbm_ctx *ctx, double out[4]);
 
-/* Algorithmic bytes one node-update of the fused step moves in and out of
- * HBM for this context's storage (populations read and written, u* read and
- * written). */
+/* Algorithmic bytes one node-update of a launch of one step moves in and out
+ * of HBM for this context's storage (populations read and written, u* read and
+ * written). A launch of two steps moves them once for both, one of many steps
+ * of a small lattice mostly finds them in the L2 cache. */
 double lbm_bytes_per_node_update(const lbm_ctx *ctx);
 
 /* Diagnostics of a state field without allocating device memory. The paper

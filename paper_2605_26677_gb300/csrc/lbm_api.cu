@@ -1267,6 +1267,16 @@ lbm_status lbm_step(lbm_ctx *c, int64_t nsteps)
     return sync_status(c);
 }
 
+lbm_status lbm_steps_per_launch(lbm_ctx *c, int64_t nsteps, int32_t *steps)
+{
+    if (!c) return fail(c, LBM_ERR_ARG, "ctx is NULL");
+    if (!steps) return fail(c, LBM_ERR_ARG, "steps is NULL");
+    if (nsteps < 1) return fail(c, LBM_ERR_ARG, "nsteps must be >= 1");
+    CK(c, cudaSetDevice(c->cfg.device));
+    *steps = !grouped_steps(c, nsteps) ? 1 : use_multi(c) ? (int32_t)std::min<int64_t>(nsteps, MULTI_STEPS) : 2;
+    return LBM_OK;
+}
+
 lbm_status lbm_step_variant(const lbm_ctx *c, int32_t *staged, int32_t *dynamic)
 {
     if (!c) return fail(nullptr, LBM_ERR_ARG, "ctx is NULL");

@@ -29,7 +29,8 @@ LBM_FB_NODE, LBM_FB_EXTRAP2 = range(2)
 EXPORTS = ["lbm_create", "lbm_destroy", "lbm_last_error", "lbm_set_material", "lbm_set_material_field",
            "lbm_set_material_field_device",
            "lbm_set_body_force",
-           "lbm_set_boundary", "lbm_set_boundary_table", "lbm_init", "lbm_init_device", "lbm_step", "lbm_step_async", "lbm_step_variant", "lbm_sync",
+           "lbm_set_boundary", "lbm_set_boundary_table", "lbm_init", "lbm_init_device", "lbm_step", "lbm_step_async",
+           "lbm_steps_per_launch", "lbm_step_variant", "lbm_sync",
            "lbm_read_state", "lbm_read_state_device", "lbm_read_displacement", "lbm_read_displacement_device",
            "lbm_read_cauchy", "lbm_diagnostics", "lbm_save", "lbm_load", "lbm_info", "lbm_profile",
            "lbm_profile_read", "lbm_bytes_per_node_update", "lbm_diagnostics_state_noalloc",
@@ -86,6 +87,7 @@ _lib.lbm_init.argtypes = [_ctx, C.c_void_p, C.c_void_p, C.c_int32]
 _lib.lbm_init_device.argtypes = [_ctx, C.c_void_p, C.c_void_p, C.c_int32]
 _lib.lbm_step.argtypes = [_ctx, C.c_int64]
 _lib.lbm_step_async.argtypes = [_ctx, C.c_int64]
+_lib.lbm_steps_per_launch.argtypes = [_ctx, C.c_int64, C.POINTER(C.c_int32)]
 _lib.lbm_step_variant.argtypes = [_ctx, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]
 _lib.lbm_sync.argtypes = [_ctx]
 _lib.lbm_read_state.argtypes = [_ctx, C.c_void_p, C.c_void_p, _dp]
@@ -271,8 +273,15 @@ def lbm_step_async(ctx, nsteps):
     _check(ctx, _lib.lbm_step_async(ctx, int(nsteps)))
 
 
+def lbm_steps_per_launch(ctx, nsteps):
+    """Steps per launch of a call of nsteps >= 1: up to 64 (a small lattice), 2 or 1."""
+    k = C.c_int32()
+    _check(ctx, _lib.lbm_steps_per_launch(ctx, nsteps, C.byref(k)))
+    return k.value
+
+
 def lbm_step_variant(ctx):
-    """{"staged": 0/1, "dynamic": 0/1}: the step-launch variant the context runs now."""
+    """{"staged": 0/1, "dynamic": 0, 1 or 4}: the variant the context runs now where a launch takes one step."""
     st, dy = C.c_int32(), C.c_int32()
     _check(ctx, _lib.lbm_step_variant(ctx, C.byref(st), C.byref(dy)))
     return {"staged": st.value, "dynamic": dy.value}

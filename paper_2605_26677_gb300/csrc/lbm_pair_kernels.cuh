@@ -4,6 +4,7 @@
 #include "lbm_bulk.cuh"
 #include "lbm_internal.h"
 #include "lbm_launch.cuh"
+#include "lbm_pair_plan.h"
 #include "lbm_step_core.cuh"
 #include "lbm_step_kernels.cuh"
 #include <type_traits>
@@ -398,14 +399,19 @@ __global__ void __launch_bounds__(128, PAIR_BLOCKS) k_pair(const __grid_constant
     unsigned flags = 0;
     // one counter: the tasks are few, and only a common order puts the long
     // ones before the short ones (over four stripes 8192^2 took 1425 instead
-    // of 1386 us a step, 4096 x 2048 clamped 200 instead of 194)
-    dyn_tasks<1>(p.a.ctr, p.a.ctr_next, p.nstrip * p.nchunk, lane, [&](int task) {
-        __syncwarp();
-        // the chunks of the bottom and top rows, whose edge rules take longest, first
-        const int i = task / p.nstrip;
-        const int chunk = i == 0 ? 0 : i == 1 ? p.nchunk - 1 : i - 1;
-        pair_task<S, LAW, VEC>(p, chunk, task - i * p.nstrip, lane, sm, flags);
-    });
+    // of 1386 us a step, 4096 x 2048 clamped 200 instead of 194). The counter
+    // sets alternate as in dyn_tasks.
+    if (blockIdx.x == 0 && threadIdx.x < DYN_STRIPES) p.a.ctr_next[threadIdx.x * DYN_CTR_STRIDE] = 0u;
+    pair_tasks(
+        4 * gridDim.x, (unsigned)(p.nstrip * p.nchunk), [&] { return lane == 0 ? atomicAdd(p.a.ctr, 1u) : 0u; },
+        [&](unsigned next) { return __shfl_sync(FULL_MASK, next, 0); },
+        [&](int task) {
+            __syncwarp();
+            // the chunks of the bottom and top rows, whose edge rules take longest, first
+            const int i = task / p.nstrip;
+            const int chunk = i == 0 ? 0 : i == 1 ? p.nchunk - 1 : i - 1;
+            pair_task<S, LAW, VEC>(p, chunk, task - i * p.nstrip, lane, sm, flags);
+        });
     flags = __reduce_or_sync(FULL_MASK, flags);
     if (flags && lane == 0) atomicOr(p.a.status, (int)flags);
 }

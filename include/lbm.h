@@ -207,16 +207,20 @@ lbm_status lbm_init_device(lbm_ctx *ctx, const double *U0_dev, const double *u0_
  * for lbm_step_async, the register kernel runs in static order. Two or more
  * steps of a small lattice (uniform material, node form of F^b) go in
  * cooperative launches of up to 64 steps each, those of a larger FP32 lattice
- * in launches of two steps, with the same results; such calls need no
- * variant and leave the choice to a later one. Where CUDA refuses a cooperative
- * launch, the steps are launches of their own. While the context's stream is
- * being captured every step is a launch of its own. A graph of captured steps
- * or read-outs works on the buffer that the state lay in at capture; it stays
- * right as long as the graphs and the calls between its replays each take an
- * even number of steps (a replay advances neither the step count nor the
- * edges' time factors).
+ * in launches of two steps where that is faster, with the same results; such
+ * calls need no variant and leave the choice to a later one. On FP32 lattices
+ * where either may be faster, the first call of at least 10 steps compares
+ * launches of one and of two steps on its own steps, and the faster is kept
+ * until the material is set or the kind of an edge changes. Where CUDA refuses
+ * a cooperative launch, the steps are launches of their own. While the
+ * context's stream is being captured every step is a launch of its own. A
+ * graph of captured steps or read-outs works on the buffer that the state lay
+ * in at capture; it stays right as long as the graphs and the calls between
+ * its replays each take an even number of steps (a replay advances neither the
+ * step count nor the edges' time factors).
  * LBM_STEP16=regs or staged, LBM_DYN=0 or 1 and LBM_DYN_STRIPES=1 or 4 in the
- * environment restrict the choice (and keep one launch per step). */
+ * environment restrict the choice (and keep one launch per step); LBM_PAIR=0
+ * or 1 has launches of two steps never, or wherever they can run. */
 lbm_status lbm_step(lbm_ctx *ctx, int64_t nsteps);
 
 /* As lbm_step without waiting; check later with lbm_sync. */

@@ -211,14 +211,11 @@ bool use_multi(const lbm_ctx *c)
     return edge_tasks <= (long long)c->multi_grid * (c->multi_block / 32);
 }
 
-// Whether k_pair takes the steps. Not where most of its tasks are those of
-// bottom and top edge rows (200000 x 8, traction: 87 us a step with it, 71
-// without; 40000 x 27: 45.3, 46.3), nor on a narrow lattice periodic in x,
-// whose wrapped columns every task copies (60 x 30000: 127, 120; 130 x 9000:
-// 60, 71).
+// Whether k_pair takes the steps
 bool use_pair(const lbm_ctx *c)
 {
-    return c->pair_grid && (yper(c) || c->L.ny >= 24) && (!xper(c) || c->L.nx >= 100);
+    if (!c->pair_grid) return false;
+    return c->pair_choice >= 0 ? c->pair_choice != 0 : c->pair_advice >= PAIR_GUESS_YES;
 }
 
 // Whether work enqueued on the context's stream is being captured (or the
@@ -312,11 +309,7 @@ cudaError_t do_pairs(lbm_ctx *c, int64_t pairs)
             p.a.g[e] = ctx_time_factor(c, e, c->step + 1);
         }
         p.a.ctr2 = c->d_ctr;
-        p.nstrip = c->pair_strips;
-        p.nchunk = c->pair_chunks;
-        p.nlong = c->pair_nlong;
-        p.hlong = c->pair_hlong;
-        p.hend = c->pair_hend;
+        p.plan = c->pair_plan;
         const cudaError_t e = launch_pair_f32(c->m.law, &p, c->pair_grid, c->st);
         if (e != cudaSuccess) return e;
         c->cur ^= 1;
@@ -377,6 +370,53 @@ lbm_status do_step(lbm_ctx *c, int64_t nsteps)
         c->cur ^= 1;
         c->step += 1;
     }
+    return LBM_OK;
+}
+
+// Whether the next call of nsteps steps begins with a comparison of k_pair
+// with the step kernel
+constexpr int COMPARE_PAIRS = 3, COMPARE_SINGLES = 4;  // launches of each in a round, the first untimed
+constexpr int COMPARE_STEPS = 2 * COMPARE_PAIRS + COMPARE_SINGLES;
+bool compare_due(lbm_ctx *c, int64_t nsteps)
+{
+    return c->pair_grid && c->pair_choice < 0 && (c->pair_advice == PAIR_GUESS_NO || c->pair_advice == PAIR_GUESS_YES) &&
+           nsteps >= COMPARE_STEPS && !c->prof && !capturing(c) && !c->captured;
+}
+
+// Steps of the call itself, one or two rounds of each kernel, timed with
+// events: the faster kernel keeps the lattice. The step kernel in the
+// dynamic order, which on these lattices is nearly always its faster one,
+// unless tune_step has chosen. *left: the call's remaining steps.
+lbm_status compare_pairs(lbm_ctx *c, int64_t *left)
+{
+    const int rounds = *left >= 2 * COMPARE_STEPS ? 2 : 1, dyn = c->dyn;
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    cudaError_t e = cudaEventCreate(&ev[0]);
+    if (e == cudaSuccess) e = cudaEventCreate(&ev[1]);
+    lbm_status s = LBM_OK;
+    float best[2] = {0.f, 0.f};  // ms a step: single, pair
+    if (c->tune_pending) c->dyn = DYN_STRIPES;
+    for (int r = 0; r < 2 * rounds && e == cudaSuccess && s == LBM_OK; ++r) {
+        const int pair = c->pair_choice = r & 1;
+        auto steps = [&](int launches) { s = do_step<float>(c, pair ? 2 * launches : launches); };
+        const int timed = (pair ? COMPARE_PAIRS : COMPARE_SINGLES) - 1;
+        float ms = 0.f;
+        steps(1);
+        e = cudaEventRecord(ev[0], c->st);
+        if (s == LBM_OK) steps(timed);
+        if (e == cudaSuccess) e = cudaEventRecord(ev[1], c->st);
+        if (e == cudaSuccess) e = cudaEventSynchronize(ev[1]);
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
+        ms /= (float)(pair ? 2 * timed : timed);
+        if (r < 2 || ms < best[pair]) best[pair] = ms;
+        *left -= pair ? 2 * COMPARE_PAIRS : COMPARE_SINGLES;
+    }
+    c->dyn = dyn;
+    c->pair_choice = e == cudaSuccess && s == LBM_OK ? best[1] < best[0] : -1;
+    for (cudaEvent_t x : ev)
+        if (x) cudaEventDestroy(x);
+    if (s != LBM_OK) return s;
+    CK(c, e);
     return LBM_OK;
 }
 
@@ -593,53 +633,39 @@ static void set_multi(lbm_ctx *c, int sms)
     c->multi_grid = (int)std::min<long long>((tasks + warps - 1) / warps, (long long)per_sm * sms);
 }
 
-// The two-step kernel (k_pair) takes the FP32 lattices that are too large for
-// k_multi. (16-bit storage would gain 1 to 5%: FP16 4096^2 314 -> 298 us a
-// step with a kernel of two nodes per lane, BF16 4096 x 2048 clamped 163.5 ->
-// 162.)
+// Plan and advice of k_pair for the present edges and law, without an earlier
+// comparison
+static void plan_pair(lbm_ctx *c)
+{
+    PairLattice l{};
+    l.nx = c->L.nx;
+    l.ny = c->L.ny;
+    l.log_law = c->m.law == LAW_LOGNH;
+    l.heavy_law = c->m.law >= LAW_MR;
+    l.xper = xper(c);
+    l.yper = yper(c);
+    l.ytraction = c->edge[EDGE_BOTTOM].kind == BC_TRACTION || c->edge[EDGE_TOP].kind == BC_TRACTION;
+    l.warps = c->pair_warps;
+    c->pair_grid = 0;
+    const int env = pair_env_choice();
+    c->pair_choice = env == 1 ? 2 : env;
+    if (!l.warps) return;
+    c->pair_plan = pair_plan(l);
+    c->pair_advice = pair_advice(l);
+    c->pair_grid = (int)std::min(((long long)c->pair_plan.nstrip * c->pair_plan.nchunk + 3) / 4, l.warps / 4LL);
+}
+
+// The two-step kernel (k_pair) takes FP32 lattices that are too large for
+// k_multi (pair_advice says which). (16-bit storage would gain 1 to 5%: FP16
+// 4096^2 314 -> 298 us a step with a kernel of two nodes per lane, BF16 4096 x
+// 2048 clamped 163.5 -> 162.)
 static void set_pair(lbm_ctx *c, int sms)
 {
-    c->pair_grid = 0;
-    if (c->multi_fn || c->cfg.storage != STORE_F32 || c->cfg.fb_mode != LBM_FB_NODE || c->m.mufield) return;
-    if (c->L.nx < 8 || c->L.ny < 8) return;
-    if (dyn_env_choice() >= 0 || stripes_env_choice() >= 0 || step16_env_choice() >= 0) return;
-    const int per_sm = pair_blocks_f32(c->m.law);
-    if (per_sm < 1) return;
-    const int ny = c->L.ny, warps = 4 * per_sm * sms;
-    c->pair_strips = (c->L.nx + PAIR_COLUMNS - 1) / PAIR_COLUMNS;
-    // Rows per task. Where tasks of 16 rows come in more than three rounds of
-    // one per warp: 16, or 24 from 16 rounds on, and 6 for about the last
-    // two rounds, which leave the warps idle for less at the launch's end (us
-    // per step, 16 rows throughout / this: 4096 x 2048 clamped 194.5 / 187,
-    // 4096^2 377 / 370, 8192^2 1386 / 1366). Smaller lattices: by a model in
-    // rows' time, a task taking one more row than it writes, its rounds
-    // whole, one long task per warp leaving the launch to its slowest warp,
-    // and the tasks of a non-periodic bottom or top row (traction Newton
-    // solves), which run first, 11 rows longer (2048 x 1024 clamped 72 with 8
-    // rows, 79 with 16; 2048^2 109 with one task per warp, 119 with 16).
-    auto rounds_of = [&](int h) { return (double)((ny + h - 1) / h) * c->pair_strips / warps; };
-    c->pair_hend = 0;
-    if (rounds_of(16) > 3.0) {
-        c->pair_hlong = rounds_of(16) > 16.0 ? 24 : 16;
-        c->pair_hend = 6;
-    } else {
-        double best = 0.0;
-        for (int h : {4, 6, 8, 12, 16, std::max(4, (ny * c->pair_strips + warps - 1) / warps)}) {
-            const double rounds = rounds_of(h);
-            double t = std::ceil(rounds) * (h + 1.0);
-            if (rounds <= 1.0 && h > 40) t *= 1.35;
-            if (!yper(c)) t = std::max(t, h + 12.0);
-            if (best == 0.0 || t < best) {
-                best = t;
-                c->pair_hlong = h;
-            }
-        }
-    }
-    const int hl = c->pair_hlong, he = c->pair_hend;
-    const int tail = he ? std::min(ny, (int)((hl == 16 ? 2.0 : 1.5) * warps / c->pair_strips * he)) : 0;
-    c->pair_nlong = he ? (ny - tail) / hl : (ny + hl - 1) / hl;
-    c->pair_chunks = c->pair_nlong + (he ? (ny - c->pair_nlong * hl + he - 1) / he : 0);
-    c->pair_grid = (int)std::min<long long>(((long long)c->pair_strips * c->pair_chunks + 3) / 4, (long long)per_sm * sms);
+    const bool can = !c->multi_fn && c->cfg.storage == STORE_F32 && c->cfg.fb_mode == LBM_FB_NODE && !c->m.mufield &&
+                     c->L.nx >= 8 && c->L.ny >= 8 && dyn_env_choice() < 0 && stripes_env_choice() < 0 &&
+                     step16_env_choice() < 0;
+    c->pair_warps = can ? 4 * pair_blocks_f32(c->m.law) * sms : 0;
+    plan_pair(c);
 }
 
 static lbm_status set_step_grid(lbm_ctx *c)
@@ -934,8 +960,10 @@ lbm_status lbm_set_boundary(lbm_ctx *c, int32_t edge, int32_t bc, const double v
     } else {
         d.profile = nullptr;
     }
+    const bool changed = c->edge[edge].kind != bc;
     c->edge[edge] = d;
     c->ghosts_dirty = true;
+    if (changed) plan_pair(c);
     return LBM_OK;
 }
 
@@ -1256,6 +1284,11 @@ lbm_status lbm_step_async(lbm_ctx *c, int64_t nsteps)
 
 lbm_status lbm_step(lbm_ctx *c, int64_t nsteps)
 {
+    if (c && nsteps > 0 && c->initialized && compare_due(c, nsteps)) {
+        lbm_status s = tlv::ctx_ready(c);
+        if (s == LBM_OK) s = compare_pairs(c, &nsteps);
+        if (s != LBM_OK) return s;
+    }
     if (c && nsteps > 0 && !grouped_steps(c, nsteps)) {
         // the context's first synchronising call that takes its steps one
         // to a launch picks the step-launch variant for the lattice (tune_step)

@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "lbm_ordered.cuh"
+#include "lbm_pair_plan.h"
 
 namespace tlv {
 
@@ -240,14 +241,12 @@ struct StepTimes {
 // (a.fin the first's input, a.fout the second's output), g1 and v1 the edge
 // data of the first (as StepTimes' rows)
 constexpr int PAIR_SIDE_ROWS = 16;
-constexpr int PAIR_VEC = 4, PAIR_COLUMNS = 30 * PAIR_VEC;  // nodes per lane, columns per strip
 template <typename R>
 struct PairArgs {
     StepArgs<R> a;
     double g1[4];
     EdgeVal<R> v1[4];
-    int nstrip, nchunk;      // strips of columns, chunks of rows
-    int nlong, hlong, hend;  // nlong chunks of hlong rows, the rest of hend
+    PairPlan plan;
 };
 
 // A batch of lattices for one persistent launch

@@ -36,6 +36,16 @@ inline int stripes_env_choice()
     return -1;
 }
 
+// LBM_PAIR=0 or 1: launches of two steps never, or wherever they can run (-1
+// when unset: pair_advice and compare_pairs choose)
+inline int pair_env_choice()
+{
+    const char *v = std::getenv("LBM_PAIR");
+    if (v && !std::strcmp(v, "0")) return 0;
+    if (v && !std::strcmp(v, "1")) return 1;
+    return -1;
+}
+
 inline int step16_env_choice()
 {
     static const int k = [] {
@@ -76,8 +86,11 @@ struct lbm_ctx {
     int grid_step = 1;
     const void *multi_fn = nullptr;  // many-steps kernel of a small lattice (set_multi), or nullptr
     int multi_block = 0, multi_grid = 0;
-    int pair_grid = 0;               // two-step kernel (set_pair); 0: not used
-    int pair_strips = 0, pair_chunks = 0, pair_nlong = 0, pair_hlong = 0, pair_hend = 0;  // as in PairArgs
+    int pair_warps = 0;              // resident warps of the two-step kernel (set_pair); 0: it cannot run
+    int pair_grid = 0;
+    tlv::PairPlan pair_plan{};       // for the present law and edges (plan_pair), as the advice
+    tlv::PairAdvice pair_advice = tlv::PAIR_NO;
+    int pair_choice = -1;            // 0 or 1: by comparison; 2 (always), 0: by LBM_PAIR; -1: by the advice
     int edge_blk_end[4] = {0, 0, 0, 0};
     std::string err;
     bool prof = false;

@@ -183,9 +183,8 @@ __device__ __forceinline__ void pair_task(const PairArgs<S> &p, int chunk, int s
     const long long plane = a.L.plane;
     const S *__restrict__ fin = static_cast<const S *>(a.fin);
     S *__restrict__ fout = static_cast<S *>(a.fout);
-    const int over = max(chunk - p.nlong, 0);  // chunks of the short kind before this one
-    const int ya = (chunk - over) * p.hlong + over * p.hend;
-    const int yb = min(ny, ya + (chunk < p.nlong ? p.hlong : p.hend));
+    int ya, yb;
+    pair_rows(p.plan, ny, chunk, ya, yb);
     const int c = (30 * strip + lane - 1) * VEC;
     const bool xper = a.kind[EDGE_LEFT] == BC_PERIODIC, yper = a.kind[EDGE_BOTTOM] == BC_PERIODIC;
     const bool ld = c <= (xper ? nx + 1 : nx);  // the lane's vector holds a column that some output needs
@@ -403,14 +402,12 @@ __global__ void __launch_bounds__(128, PAIR_BLOCKS) k_pair(const __grid_constant
     // sets alternate as in dyn_tasks.
     if (blockIdx.x == 0 && threadIdx.x < DYN_STRIPES) p.a.ctr_next[threadIdx.x * DYN_CTR_STRIDE] = 0u;
     pair_tasks(
-        4 * gridDim.x, (unsigned)(p.nstrip * p.nchunk), [&] { return lane == 0 ? atomicAdd(p.a.ctr, 1u) : 0u; },
+        4 * gridDim.x, (unsigned)(p.plan.nstrip * p.plan.nchunk), [&] { return lane == 0 ? atomicAdd(p.a.ctr, 1u) : 0u; },
         [&](unsigned next) { return __shfl_sync(FULL_MASK, next, 0); },
         [&](int task) {
             __syncwarp();
-            // the chunks of the bottom and top rows, whose edge rules take longest, first
-            const int i = task / p.nstrip;
-            const int chunk = i == 0 ? 0 : i == 1 ? p.nchunk - 1 : i - 1;
-            pair_task<S, LAW, VEC>(p, chunk, task - i * p.nstrip, lane, sm, flags);
+            const int i = task / p.plan.nstrip;
+            pair_task<S, LAW, VEC>(p, pair_chunk(p.plan, i), task - i * p.plan.nstrip, lane, sm, flags);
         });
     flags = __reduce_or_sync(FULL_MASK, flags);
     if (flags && lane == 0) atomicOr(p.a.status, (int)flags);

@@ -374,19 +374,19 @@ __device__ __forceinline__ void pair_task(const PairArgs<S> &p, int chunk, int s
 }
 
 // Two steps in one pass: f*^n is read, f*^{n+1} lives in registers and shared
-// memory only, f*^{n+2} is written, and u* moves once for both steps, 112
-// instead of 224 bytes of HBM traffic per node and step. A warp goes down a
-// strip of columns row by row (pair_task); the strips overlap by a lane on
-// either side and the row chunks by a row, 7% and 6 to 12% of reads done
+// memory only, f*^{n+2} is written, and u* moves once for both steps: 112
+// instead of 224 bytes per node and step, 122 measured (4096^2). A warp goes
+// down a strip of columns row by row (pair_task); the strips overlap by a lane
+// on either side and the row chunks by a row, 7% and 4 to 12% of reads done
 // twice. The warps need nothing of one another. Its next row is copied to
 // shared memory in the background of the current one (without that copy 1591
 // instead of 1406 us a step on 8192^2, with u* read when it is needed and its
 // velocities widened on the FP64 pipe 1580). Barriers that keep the warps of
 // a block on the same row made it slower (1756). The same bits as two
 // launches of k_step; us per step, k_step / k_pair: 8192^2 periodic 2145 /
-// 1366, 4096 x 2048 clamped 278 / 187, 2048^2 periodic 144 / 109. What binds it now
-// is the latency of a warp's own chain at eight warps per SM (32% of issue
-// slots) and HBM at 5.3 TB/s; with the collisions taken out it moves its
+// 1366, 4096 x 2048 clamped 284 / 187, 2048^2 periodic 149 / 106. What binds it now
+// is the latency of a warp's own chain at eight warps per SM (33% of issue
+// slots) and HBM at 5.5 TB/s; with the collisions taken out it moves its
 // data at 5.7 TB/s.
 template <typename S, int LAW, int VEC>
 __global__ void __launch_bounds__(128, PAIR_BLOCKS) k_pair(const __grid_constant__ PairArgs<S> p)

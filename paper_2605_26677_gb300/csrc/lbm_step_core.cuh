@@ -15,8 +15,8 @@ struct alignas(sizeof(T) * N) Pack {
 
 #define FULL_MASK 0xffffffffu
 
-// What changes from one step of a launch to the next: the population buffers
-// and the edges' time factors (nullptr: StepArgs::g)
+// The population buffers of a step and the device copy of its edges' time
+// factors (nullptr: those of StepArgs::g, as k_pair has it throughout)
 struct StepIO {
     const void *fin;
     void *fout;

@@ -202,13 +202,19 @@ lbm_status record(lbm_ctx *c, std::vector<cudaEvent_t> &v)
 // whose rows mostly hold a node of a non-periodic side edge: k_multi applies
 // that edge's rule in the node's own warp, the FP64 step kernel 32 of them at
 // a time from a queue, which pays once warps take several rows each (26 x
-// 5535, traction: 157 us a step there, 165 with k_multi).
+// 5535, traction: 157 us a step there, 165 with k_multi), nor with the long
+// Newton solves of MR, Yeoh and Gent on traction sides alone, where most warps
+// have one beside other rounds (124 x 502 MR: 91, 128).
 bool use_multi(const lbm_ctx *c)
 {
     if (!c->multi_fn) return false;
     if (c->cfg.storage != STORE_F64 || xper(c)) return true;
-    const long long edge_tasks = (long long)c->L.ny * std::min(2, (c->L.nx + 31) / 32);
-    return edge_tasks <= (long long)c->multi_grid * (c->multi_block / 32);
+    const long long warps = (long long)c->multi_grid * (c->multi_block / 32), segs = (c->L.nx + 31) / 32;
+    const long long edge_tasks = c->L.ny * std::min(2LL, segs);
+    if (edge_tasks > warps) return false;
+    auto traction = [&](int e, int f) { return c->edge[e].kind == BC_TRACTION || c->edge[f].kind == BC_TRACTION; };
+    return !(c->m.law >= LAW_MR && traction(EDGE_LEFT, EDGE_RIGHT) && !traction(EDGE_BOTTOM, EDGE_TOP) &&
+             c->L.ny * segs > warps && 4 * edge_tasks > 3 * warps);
 }
 
 // Whether k_pair takes the steps
@@ -624,13 +630,13 @@ static void set_multi(lbm_ctx *c, int sms)
     case STORE_F16: fn = multi_kernel_f16(c->m.law); break;
     default: fn = multi_kernel_f32(c->m.law); break;
     }
-    // few tasks: one warp to a block, so that they spread over the SMs
     const long long tasks = (long long)c->L.ny * ((c->L.nx + 31) / 32);
-    const int warps = (int)std::min<long long>(MULTI_WARPS, std::max<long long>(1, (tasks + sms - 1) / sms));
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * warps, 0) != cudaSuccess || per_sm < 1) return;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * MULTI_WARPS, 0) != cudaSuccess || per_sm < 1)
+        return;
+    const MultiGrid g = multi_grid(tasks, sms, per_sm);
     c->multi_fn = fn;
-    c->multi_block = 32 * warps;
-    c->multi_grid = (int)std::min<long long>((tasks + warps - 1) / warps, (long long)per_sm * sms);
+    c->multi_block = 32 * g.warps;
+    c->multi_grid = g.blocks;
 }
 
 // Plan and advice of k_pair for the present edges and law, without an earlier

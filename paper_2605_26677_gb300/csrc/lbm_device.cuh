@@ -21,6 +21,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include "lbm_multi_plan.h"
 #include "lbm_ordered.cuh"
 #include "lbm_pair_plan.h"
 
@@ -228,9 +229,6 @@ struct EdgeVal {
 // Edge data of the steps of one many-steps launch (a kernel argument): the
 // time factors, and the values of edges without a profile
 constexpr int MULTI_STEPS = 64;
-constexpr int MULTI_WARPS = 8;  // warps per block at most (4: more blocks meet at the barrier,
-                                // 512^2 FP32 8.7 against 8.0 us a step; 16: 7.7, but FP64 512^2 138
-                                // against 113)
 template <typename R>
 struct StepTimes {
     double g[MULTI_STEPS][4];

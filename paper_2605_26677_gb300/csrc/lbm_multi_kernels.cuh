@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(32 * MULTI_WARPS) k_multi(const __grid_constan
     const int gw = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     const int nw = gridDim.x * (blockDim.x >> 5);
     const int nseg = (a.L.nx + 31) / 32, ntask = a.L.ny * nseg;
+    const bool twist = multi_twist(nseg, nw);
     unsigned flags = 0;
     void *const f0 = const_cast<void *>(a.fin);
     for (int s = 0; s < nsteps; ++s) {
@@ -102,7 +103,7 @@ __global__ void __launch_bounds__(32 * MULTI_WARPS) k_multi(const __grid_constan
         void *to = (s & 1) ? f0 : a.fout;
         for (int task = gw; task < ntask; task += nw) {
             int y, seg;
-            task_coords(task, nseg, a.L.ny, y, seg);
+            multi_coords(task, nseg, a.L.ny, twist, y, seg);
             const int x = seg * 32 + lane;
             if (x < a.L.nx) node_step<S, LAW>(a, tab, s, from, to, x, y, flags);
         }

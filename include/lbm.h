@@ -205,10 +205,11 @@ lbm_status lbm_init_device(lbm_ctx *ctx, const double *U0_dev, const double *u0_
  * state untouched, and the fastest is kept for the context's life (the
  * trials take a u*-sized scratch allocation while they run). Until then, and
  * for lbm_step_async, the register kernel runs in static order. Two or more
- * steps of a small lattice (uniform material, node form of F^b) go in
- * cooperative launches of up to 64 steps each, those of a larger FP32 lattice
- * in launches of two steps where that is faster, with the same results; such
- * calls need no variant and leave the choice to a later one. On FP32 lattices
+ * steps (three in 16 bits without edges) of a small lattice (uniform material,
+ * node form of F^b) go in cooperative launches of up to 64 steps each, those
+ * of a larger FP32 lattice in launches of two steps where that is faster, with
+ * the same results; such calls need no variant and leave the choice to a later
+ * one. On FP32 lattices
  * where either may be faster, the first call of at least 10 steps compares
  * launches of one and of two steps on its own steps, and the faster is kept
  * until the material is set or the kind of an edge changes. Where CUDA refuses

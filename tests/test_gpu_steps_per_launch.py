@@ -24,3 +24,15 @@ def test_steps_per_launch(lbm, monkeypatch, nx, ny, storage, want):  # noqa: F81
     with pytest.raises(lbm.LbmError):
         lbm.lbm_steps_per_launch(L.ctx, 0)
     L.close()
+
+
+@pytest.mark.parametrize("storage,periodic,want", [(2, True, 1), (3, True, 1), (2, False, 2), (1, True, 2)])
+def test_two_steps_of_a_16_bit_lattice(lbm, storage, periodic, want):  # noqa: F811
+    L = lbm.Lattice(300, 300, c=6.0, omega=1.9, storage=storage)
+    lbm.lbm_set_material(L.ctx, 1, [1.5, 0.75])
+    if not periodic:
+        for e in (0, 1):
+            lbm.lbm_set_boundary(L.ctx, e, lbm.LBM_BC_VELOCITY)
+    assert lbm.lbm_steps_per_launch(L.ctx, 2) == want
+    assert lbm.lbm_steps_per_launch(L.ctx, 3) == 3
+    L.close()
